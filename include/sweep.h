@@ -54,11 +54,19 @@ enum { SWEEP_FACE_BOUNDARY = 1, SWEEP_FACE_PERIODIC = 2 };
 
 /* Schedules of the batched sweep kernel. */
 enum {
-    SWEEP_SCHED_AUTO = 0,     /* pick by a one-time timing of LEVEL vs DATAFLOW per context */
+    SWEEP_SCHED_AUTO = 0,     /* narrow levels: one block per direction (below); else a one-time timing of LEVEL vs
+                                 DATAFLOW per context */
     SWEEP_SCHED_LEVEL = 1,    /* persistent kernel, grid barrier between wavefront levels */
     SWEEP_SCHED_DATAFLOW = 2, /* persistent kernel, no barriers: each task waits (bounded) for its upwind values */
     SWEEP_SCHED_PLAIN = 3     /* plain FP64 path: one kernel launch per (direction, level), no batching */
 };
+
+/* AUTO, with lanes_per_task, packets_per_step, block_threads and blocks_per_sm left at 0, op_format not LINES and
+ * geometry_only 0, sweeps narrow levels (up to 256 tasks per direction and level on average, in FP64 512) with one
+ * block per direction: barriers between the levels of that direction only, and the operator in a stream of its
+ * own order. Values of 1, 2 or 4 groups (transposed: 2 or 4 split groups), rows of up to 64 face sides, in FP64 the
+ * BALANCE law. sweep_stats then reports schedule_used LEVEL, kernel_used PACKED, lanes_used and
+ * blocks_per_sm_used 1. */
 
 /* Absorption laws of the cell update (transport scheme (a) of Sec. 2.6, outflow = non-absorbed inflow
  * plus source; F_in = the inflow flux, P = the projected outflow area, tau = kappa_t V / P):
@@ -68,7 +76,7 @@ enum {
  *            removed flux; with kappa_a = 0 the scattered fraction is 1 - exp(-kappa_s V / P), the
  *            scattering law of Sec. 3.3. Forward solves only (the adjoint takes BALANCE). In FP32 EXP
  *            runs over the packed operator (1, 2 or 4 groups; otherwise, and in FP64, in the kernels that
- *            read the mesh rows), on the DATAFLOW schedule when the schedule is AUTO (no autotuning),
+ *            read the mesh rows), on the DATAFLOW schedule when the schedule is AUTO and the levels are wide (no autotuning),
  *            and keeps one more [D][N][G] array. */
 enum { SWEEP_LAW_BALANCE = 0, SWEEP_LAW_EXP = 1 };
 
@@ -139,7 +147,8 @@ typedef struct {
     int32_t sweep_launches;    /* batched-sweep kernel launches timed in t_ms[2] */
     int32_t schedule_used;     /* SWEEP_SCHED_* that ran */
     int32_t kernel_launches;   /* all kernels this call launched (including the autotuner's) */
-    int32_t lanes_used;        /* lanes per task of the batched sweep that ran (packed operator: 32 x packets per step) */
+    int32_t lanes_used;        /* lanes per task of the batched sweep that ran (packed operator: 32 x packets per step, or 1 with
+                                  one block per direction) */
     int32_t threads_used;      /* threads per block of the batched sweep that ran */
     int32_t blocks_per_sm_used;/* resident blocks per SM it was launched with (0 = maximum) */
     int32_t kernel_used;       /* SWEEP_KERNEL_* form of the batched sweep that ran last */

@@ -83,6 +83,9 @@ struct sweep_ctx {
 
 namespace {
 
+// internal schedule: one block per direction (dirsweep.cu)
+constexpr int SCHED_DIR = 100;
+
 sweep_status cuda_status(sweep_ctx* c, cudaError_t e, const char* what) {
     if (e == cudaSuccess) return SWEEP_OK;
     c->err = std::string(what) + ": " + cudaGetErrorString(e);
@@ -120,6 +123,10 @@ void free_levels(Levels& L) {
         dfree(P->pk); dfree(P->meta); dfree(P->lev_pk); dfree(P->grp); dfree(P->lev_grp); dfree(P->cnt);
         dfree(P->off); dfree(P->scan); dfree(P->flag);
     }
+    for (DirOp* P : {&L.dop, &L.dopt}) {
+        dfree(P->E); dfree(P->C); dfree(P->meta);
+    }
+    dfree(L.dir_ws);
     dfree(L.lfill);
     dfree(L.dc_mask); dfree(L.dc_inm); dfree(L.dc_share32); dfree(L.dc_share64);
     L = Levels();
@@ -153,12 +160,19 @@ int dir_bits(int nd) {
     return b;
 }
 
+// the operators belong to levels that are about to change
+void drop_operators(Levels& L) {
+    L.op_valid = false;
+    L.pkt.valid = false;
+    L.dop.valid = false;
+    L.dopt.valid = false;
+}
+
 sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
     const int64_t N = c->mesh.N;
     if (L.nd == nd && L.raw && L.d0 == d0) {
         L.valid = false;
-        L.op_valid = false;
-        L.pkt.valid = false;
+        drop_operators(L);
         return SWEEP_OK;
     }
     free_levels(L);
@@ -170,8 +184,6 @@ sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
     if ((uint64_t)N > (uint64_t)L.cmask + 1ull) return bad(c, "n_cells too large for the number of directions");
     L.task_cap = N * (int64_t)nd + 32 * (N + 2);
     CK(cudaMalloc(&L.raw, sizeof(uint32_t) * L.task_cap), "alloc task list");
-    CK(cudaMalloc(&L.task, sizeof(uint32_t) * L.task_cap), "alloc task list");
-    CK(cudaMalloc(&L.trec, sizeof(int4) * L.task_cap), "alloc task records");
     CK(cudaMalloc(&L.info, sizeof(int4) * N * nd), "alloc classification");
     CK(cudaMalloc(&L.level, sizeof(int32_t) * N * nd), "alloc levels");
     CK(cudaMalloc(&L.lvl_cnt, sizeof(int32_t) * (N + 2)), "alloc level counts");
@@ -353,6 +365,9 @@ sweep_status run_sweep(sweep_ctx* c, const Levels& L, int precision, int schedul
                 if (b1 > b0) CKL(launch_plain_level(a, b0, b1, c->st), "plain sweep");
             }
         }
+    } else if (schedule == SCHED_DIR) {
+        c->last_kernel = SWEEP_KERNEL_PACKED;
+        CKL(launch_sweep_dir(a, a.reverse ? L.dopt : L.dop, pk_mode(a), c->sms, c->st), "sweep launch");
     } else {
         const int fmt = a.pk ? OPF_PACKETS : (a.op ? OPF_LINES : OPF_NONE);
         // without an assembled operator the adjoint, the EXP law and scheme (b) run in the generic kernel
@@ -468,8 +483,8 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
     int fmt = (prec == 32 && c->lev.op_valid && !o.geometry_only) ? c->lev.op_format : OPF_NONE;
     if (o.law && fmt == OPF_LINES) fmt = OPF_NONE;  // the EXP law: packets or the mesh rows
     const bool generic = fmt == OPF_NONE && (o.law || c->lev.transport > 0);
-    int per_sm = sweep_occupancy(prec, G, threads, c->lev.nd, lanes, generic ? 1 : 0, fmt,
-                                 o.law ? PK_EXP : PK_BALANCE);
+    int per_sm = sched == SCHED_DIR ? 1 : sweep_occupancy(prec, G, threads, c->lev.nd, lanes, generic ? 1 : 0, fmt,
+                                                          o.law ? PK_EXP : PK_BALANCE);
     if (per_sm < 1) return bad(c, "sweep kernel does not fit on an SM");
     if (bpsm > 0 && bpsm < per_sm) per_sm = bpsm;
     const int period = pbc ? 4 : 2;
@@ -500,7 +515,13 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
         a.debug_stall = 0;
         if (prec == 32) a.bc = bc32;
         a.lanes = lanes;
-        if ((e = launch_sweep(a, prec, c->sms * per_sm, threads, gs, &kid))) return e;
+        if (sched == SCHED_DIR) {
+            kid = SWEEP_KERNEL_PACKED;
+            e = launch_sweep_dir(a, c->lev.dop, pk_mode(a), c->sms, gs);
+        } else {
+            e = launch_sweep(a, prec, c->sms * per_sm, threads, gs, &kid);
+        }
+        if (e) return e;
         if ((e = cudaEventRecordWithFlags(ev[1], gs, cudaEventRecordExternal))) return e;
         if (scat) {
             if ((e = launch_tally(prec, o.law ? c->Imean : b.I[cur], N, G, D, 0, c->w64, c->wsum, c->mesh.vol, c->ka,
@@ -1008,14 +1029,68 @@ sweep_status ensure_operator(sweep_ctx* c, Levels& L, const sweep_opts* o, int p
     return SWEEP_OK;
 }
 
+// Whether a sweep with these options may run with one block per direction: the schedule and its parameters
+// left to the library, values of 1, 2 or 4 groups (transposed: 2 or 4 split groups), and in FP64 the
+// BALANCE law (the EXP law reads the mesh rows).
+bool dir_wanted(const sweep_opts* o, int prec, int width, bool transposed) {
+    if (!o || o->schedule != SWEEP_SCHED_AUTO || o->geometry_only || o->op_format == SWEEP_OP_LINES || o->lanes_per_task ||
+        o->packets_per_step || o->block_threads || o->blocks_per_sm || o->debug_stall)
+        return false;
+    if (prec == 64 && o->law != SWEEP_LAW_BALANCE) return false;
+    return width == 2 || width == 4 || (width == 1 && !transposed);
+}
+
+// The per-direction operator of the cached levels for values of `width` numbers, built once per levelisation
+// and width. P.valid stays false where it does not apply or does not fit in device memory.
+sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int prec, int width, float* t_ms) {
+    const int rb = prec == 64 ? 8 : 4;
+    if (P.valid && P.real_bytes == rb && P.GC == width) return SWEEP_OK;
+    P.valid = false;
+    ScopedEvent e0, e1;
+    cudaEventRecord(e0, c->st);
+    bool ok = false;
+    CK(dir_plan(c->mesh, L, P, transposed, rb, width, c->om64, c->om32, c->om32lo, c->sms, c->st, &ok), "plan operator");
+    auto grow = [&](unsigned char*& p, int64_t& cap, int64_t need) {
+        if (need <= cap) return true;
+        dfree(p);
+        cap = 0;
+        const int64_t n = need + need / 16 + 256;
+        if (!op_fits((size_t)n) || cudaMalloc(&p, (size_t)n) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+            return false;
+        }
+        cap = n;
+        return true;
+    };
+    ok = ok && grow(P.E, P.e_cap, P.e_bytes) && grow(P.C, P.c_cap, P.c_bytes);
+    if (ok) {
+        CK(dir_write(P, c->st), "write operator");
+        P.valid = true;
+    }
+    c->launches += P.launches;
+    cudaEventRecord(e1, c->st);
+    CK(cudaEventSynchronize(e1), "assemble operator");
+    float ms = 0;
+    cudaEventElapsedTime(&ms, e0, e1);
+    if (t_ms) *t_ms += ms;
+    return SWEEP_OK;
+}
+
+// the level-major task list of the cached levels
+sweep_status ensure_merged(sweep_ctx* c, Levels& L) {
+    if (!L.merged) c->launches += 4;
+    CK(merge_levels(c->mesh, L, c->st), "merge levels");
+    return SWEEP_OK;
+}
+
 // Levels of every direction in the dependency graph of the requested transport scheme (without options:
 // whatever scheme is cached, else scheme (a)).
 sweep_status ensure_levels(sweep_ctx* c, const sweep_opts* o, float* t1, float* t2) {
     const int tr = o ? o->transport : (c->lev.valid ? c->lev.transport : 0);
     if (c->lev.valid && !(o && o->relevel) && c->lev.nd == c->D && c->lev.d0 == 0 && c->lev.transport == tr)
         return SWEEP_OK;
-    c->lev.op_valid = false;
-    c->lev.pkt.valid = false;
+    drop_operators(c->lev);
     return run_levelise(c, c->lev, 0, c->D, budget_of(o), t1, t2, tr);
 }
 
@@ -1183,8 +1258,18 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     float tc = 0, tl = 0, top = 0;
     sweep_status s = ensure_levels(c, &o, &tc, &tl);
     if (s != SWEEP_OK) return s;
-    s = ensure_operator(c, c->lev, &o, prec, &top);
-    if (s != SWEEP_OK) return s;
+    bool by_dir = !plain && dir_wanted(&o, prec, c->G, false);
+    if (by_dir) {
+        s = ensure_dir(c, c->lev, c->lev.dop, false, prec, c->G, &top);
+        if (s != SWEEP_OK) return s;
+        by_dir = c->lev.dop.valid;
+    }
+    if (!by_dir) {
+        s = ensure_merged(c, c->lev);
+        if (s != SWEEP_OK) return s;
+        s = ensure_operator(c, c->lev, &o, prec, &top);
+        if (s != SWEEP_OK) return s;
+    }
     S.t_ms[0] = tc;
     S.t_ms[1] = tl;
     S.t_ms[5] = top;
@@ -1220,6 +1305,11 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     int sched = o.schedule, threads = o.block_threads ? o.block_threads : 256;
     int lanes = o.lanes_per_task ? o.lanes_per_task : 4;
     int bpsm = o.blocks_per_sm;
+    if (by_dir) {
+        sched = SCHED_DIR;
+        threads = 64 * c->lev.dop.W + 64;
+        lanes = bpsm = 1;
+    }
     // the EXP law: no tuning, the dataflow schedule (packets: two per warp step)
     if (!plain && sched == SWEEP_SCHED_AUTO && o.law) sched = SWEEP_SCHED_DATAFLOW;
     if (!plain && sched == SWEEP_SCHED_AUTO) {
@@ -1235,7 +1325,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         if (!o.lanes_per_task) lanes = tl;
     }
     // the packed operator's kernel has whole warps per packet: lanes = 32 x packets per warp step
-    const bool packed = prec == 32 && !o.geometry_only && c->lev.op_valid && c->lev.op_format == OPF_PACKETS;
+    const bool packed = !by_dir && prec == 32 && !o.geometry_only && c->lev.op_valid && c->lev.op_format == OPF_PACKETS;
     if (!plain && packed) {
         if (o.packets_per_step) lanes = 32 * o.packets_per_step;
         else if (lanes < 32) lanes = 64;
@@ -1261,7 +1351,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
             std::swap(c->jn, c->jn1);
         }
     }
-    S.schedule_used = sched;
+    S.schedule_used = by_dir ? (int)SWEEP_SCHED_LEVEL : sched;
     S.lanes_used = lanes;
     S.threads_used = threads;
     S.blocks_per_sm_used = bpsm;
@@ -1528,20 +1618,34 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     const int pk_lanes = o.packets_per_step ? 32 * o.packets_per_step : (tuned[0] && tuned[2] >= 32 ? tuned[2] : 64);
     const int pk_bpsm = o.blocks_per_sm ? o.blocks_per_sm : (tuned[0] ? tuned[3] : 0);
     int n_sweeps = it_fwd, it_adj = 0;
+    bool fwd_dir = false, tr_dir = false;
     bool conv_adj = true;
     double res_adj = 0.0;
     for (int d0 = 0; d0 < D; d0 += B) {
         const int nb = (D - d0) < B ? (D - d0) : B;
         Levels* L;
         float a1 = 0, a2 = 0;
+        // one block per direction where the schedule is the library's choice: the forward recompute and the
+        // transposed sweep each on their own
+        fwd_dir = tr_dir = false;
         if (nb == D) {
-            s = ensure_levels(c, &o, &a1, &a2);
-            if (s == SWEEP_OK) s = ensure_operator(c, c->lev, &o, prec, &tasm);
-            if (s == SWEEP_OK) s = ensure_transposed(c, c->lev, &o, prec, &tasm);
             L = &c->lev;
+            s = ensure_levels(c, &o, &a1, &a2);
+            if (s == SWEEP_OK && !plain && !coupled && dir_wanted(&o, prec, G, false)) {
+                s = ensure_dir(c, *L, L->dop, false, prec, G, &tasm);
+                fwd_dir = L->dop.valid;
+            }
+            if (s == SWEEP_OK && !plain && dir_wanted(&o, prec, 2 * G, true)) {
+                s = ensure_dir(c, *L, L->dopt, true, prec, 2 * G, &tasm);
+                tr_dir = L->dopt.valid;
+            }
+            if (s == SWEEP_OK && !(tr_dir && (fwd_dir || coupled))) s = ensure_merged(c, *L);
+            if (s == SWEEP_OK && !fwd_dir && !coupled) s = ensure_operator(c, *L, &o, prec, &tasm);
+            if (s == SWEEP_OK && !tr_dir) s = ensure_transposed(c, *L, &o, prec, &tasm);
         } else {
             s = run_levelise(c, c->adj_lev, d0, nb, budget_of(&o), &a1, &a2);
             L = &c->adj_lev;
+            if (s == SWEEP_OK) s = ensure_merged(c, *L);
         }
         if (s != SWEEP_OK) return s;
         tcl += a1;
@@ -1557,8 +1661,8 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
             int pI = !signI;
             SweepArgs a = make_args(c, *L, prec, cm, c->adjI, nullptr, G, pI, 0, 0, &o);
             a.debug_stall = 0;
-            s = run_sweep(c, *L, prec, plain ? SWEEP_SCHED_PLAIN : sched, threads, a.pk ? pk_lanes : lanes,
-                          a.pk ? pk_bpsm : 0, a, bc32, &t_sweep);
+            s = run_sweep(c, *L, prec, plain ? SWEEP_SCHED_PLAIN : (fwd_dir ? SCHED_DIR : sched), threads,
+                          a.pk ? pk_lanes : lanes, a.pk ? pk_bpsm : 0, a, bc32, &t_sweep);
             if (s != SWEEP_OK) return s;
             signI = pI;
             ++n_sweeps;
@@ -1574,8 +1678,8 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
             SweepArgs r = make_args(c, *L, prec, cm, lbuf[kl], pbc ? lbuf[1 - kl] : nullptr, 2 * G, pL, 1, 0, &o);
             r.debug_stall = 0;
             float t1 = 0.f;
-            s = run_sweep(c, *L, prec, plain ? SWEEP_SCHED_PLAIN : sched, threads, r.pk ? pk_lanes : lanes,
-                          r.pk ? pk_bpsm : 0, r, nullptr, &t1);
+            s = run_sweep(c, *L, prec, plain ? SWEEP_SCHED_PLAIN : (tr_dir ? SCHED_DIR : sched), threads,
+                          r.pk ? pk_lanes : lanes, r.pk ? pk_bpsm : 0, r, nullptr, &t1);
             t_sweep += t1;
             t_tr += t1;
             if (s != SWEEP_OK) return s;
@@ -1635,7 +1739,7 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
         S.depth_mean = Ld.depth.empty() ? 0.0 : dsum / Ld.depth.size();
     }
     S.updates_per_s = ttot > 0 ? S.updates / (ttot * 1e-3) : 0.0;
-    S.schedule_used = plain ? SWEEP_SCHED_PLAIN : sched;
+    S.schedule_used = plain ? SWEEP_SCHED_PLAIN : (tr_dir ? (int)SWEEP_SCHED_LEVEL : sched);
     S.kernel_used = c->last_kernel;
     S.kernel_launches = (int32_t)(c->launches - launches0);
     if (stats) *stats = S;
@@ -1791,8 +1895,7 @@ sweep_status sweep_rotate_directions(sweep_ctx* c, const double* R, int64_t n_qu
     CK(cudaMemcpy(c->om32, o32.data(), sizeof(float4) * D, cudaMemcpyHostToDevice), "upload directions");
     CK(cudaMemcpy(c->om32lo, o32lo.data(), sizeof(float4) * D, cudaMemcpyHostToDevice), "upload directions");
     c->lev.valid = false;
-    c->lev.op_valid = false;
-    c->lev.pkt.valid = false;
+    drop_operators(c->lev);
     c->adj_lev.valid = false;
     return SWEEP_OK;
 }

@@ -37,7 +37,8 @@ constexpr uint32_t PK_BOUNDARY = 0x80000000u;  // source-index bit of a boundary
 // transposed balance of the adjoint sweep (source scaled by the direction weight)
 enum { PK_BALANCE = 0, PK_EXP = 1, PK_TRANSPOSED = 2 };
 // forms of the assembled operator
-enum { OPF_NONE = 0, OPF_LINES = 1, OPF_PACKETS = 2 };
+enum { OPF_NONE = 0, OPF_LINES = 1, OPF_PACKETS = 2, OPF_DIR = 3 };
+
 
 struct GridBar {
     unsigned count;
@@ -282,6 +283,26 @@ __device__ __forceinline__ float side_weight(const int4& r, const float4& lo, co
     return fabsf(dot_comp(__int_as_float(r.y), __int_as_float(r.z), __int_as_float(r.w), lo, om, oml));
 }
 
+// The EXP law of one cell and group in the FP32 operator kernels (outgoing intensity and cell mean; see
+// exp_update in sweep.cu): one expf and two fast reciprocals, selects instead of branches. The mean factor
+// f = (1 - exp(-tau)) / tau is taken from its Taylor series sum_k (-tau)^k / (k+1)! (seven terms,
+// truncation below 2e-9) where 1 - exp(-tau) would cancel (tau < 1/4), and directly above.
+__device__ __forceinline__ void exp_update_lanes(float fin, float q, float ktv, float P, float& out, float& mean) {
+    const float rP = __fdividef(1.f, P), rK = __fdividef(1.f, ktv);
+    const float tau = ktv * rP;
+    const float e = expf(-tau);
+    const float s = -tau;
+    float ft = fmaf(s, 1.f / 5040.f, 1.f / 720.f);
+    ft = fmaf(s, ft, 1.f / 120.f);
+    ft = fmaf(s, ft, 1.f / 24.f);
+    ft = fmaf(s, ft, 1.f / 6.f);
+    ft = fmaf(s, ft, 0.5f);
+    ft = fmaf(s, ft, 1.f);
+    const float f = tau < 0.25f ? ft : (1.f - e) * P * rK;
+    const float stay = (q + fin) * rK;  // P = 0: no outflow
+    out = P > 0.f ? fmaf(e, fin, q) * rP : stay;
+    mean = P > 0.f ? fin * rP * f : stay;
+}
 // Grid-wide barrier for persistent cooperative kernels, with a bounded wait.
 // Returns false (and sets *err) if the wait gave up or another block reported an error.
 __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, long long budget, int* err) {
@@ -356,8 +377,38 @@ struct PackedOp {
     bool valid = false;          // transposed operator: built for the current levels
 };
 
+// Streams of one direction in the per-direction operator (dirsweep.cu).
+struct DirMeta {
+    int64_t e_base, e_bytes, c_base, c_bytes;
+    int rounds, pad;
+};
+
+// The operator with one block per direction: entry and control streams of every direction, and the
+// shared-memory plan they were written for.
+struct DirOp {
+    unsigned char *E = nullptr, *C = nullptr;
+    int64_t e_cap = 0, c_cap = 0;      // bytes allocated
+    int64_t e_bytes = 0, c_bytes = 0;  // bytes of the current plan
+    DirMeta* meta = nullptr;           // [nd]
+    size_t meta_bytes = 0;             // of meta and rtab (one allocation)
+    uint2* rtab = nullptr;             // [nd][rstride] offsets of every round
+    int rstride = 0;
+    int real_bytes = 0, GC = 0;        // values it was planned for
+    int W = 0, R = 0, A = 0, Fs = 0;   // slices per round, ring places, rounds fetched ahead, far sources per stage
+    int form = 0;                      // of the kernel: narrow or wider levels
+    uint32_t e_slot = 0, c_slot = 0, off_cm = 0, off_c = 0, off_e = 0, smem = 0;
+    int launches = 0;                  // kernels of the last build
+    std::vector<char> args;            // build arguments kept between plan and write
+    bool valid = false;                // written for the current levels
+};
+
 struct Levels {
     bool valid = false;
+    bool by_dir = false;         // levelised one direction per block: per-direction level lists are there
+    bool merged = false;         // the level-major task list of all directions is there
+    DirOp dop, dopt;             // per-direction operator, forward and transposed
+    void* dir_ws = nullptr;      // tables their builds work in
+    size_t dir_ws_bytes = 0;
     int d0 = 0, nd = 0;
     int cshift = 0;
     uint32_t cmask = 0;
@@ -463,6 +514,12 @@ cudaError_t pack_plan(const DevMesh& m, const Levels& L, PackedOp& P, bool trans
                       const float4* om32_all, const float4* om32lo_all, cudaStream_t st, int64_t* n_pk);
 cudaError_t pack_write(const DevMesh& m, const Levels& L, PackedOp& P, bool transposed, const double* om64_all,
                        const float4* om32_all, const float4* om32lo_all, cudaStream_t st);
+// the level-major task list of levels made by direction (what every sweep but the per-direction one reads)
+cudaError_t merge_levels(const DevMesh& m, Levels& L, cudaStream_t st);
+cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int real_bytes, int GC, const double* om64_all,
+                     const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok);
+cudaError_t dir_write(DirOp& P, cudaStream_t st);
+cudaError_t launch_sweep_dir(const SweepArgs& a, const DirOp& P, int mode, int sms, cudaStream_t st);
 cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const float4* om32_all,
                      const float4* om32lo_all, int dev_sms, GridBar* bar, int* err, long long budget,
                      int64_t* d_scratch, cudaStream_t st, float* t_classify, float* t_levelise, std::string* msg);

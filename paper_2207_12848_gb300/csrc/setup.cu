@@ -695,7 +695,7 @@ struct DirLevArgs {
     const uint64_t* dc_mask; // scheme (b): [N][nd] chosen outflow sides (release only those), or null
     int32_t* level;          // [nd][N]: minus the unsolved upwind cells, then the level
     uint32_t* dlist;         // [nd][N] cells of each direction in level order; level 0 from the classification
-    const int32_t* n0;       // [nd] level-0 sizes
+    int32_t* n0;             // [nd] level-0 sizes; then the cells levelised (fewer than N: a cycle)
     int32_t* dcnt;           // [nd][cap] cells on each level
     int32_t* dbase;          // [nd][cap] start of each level in dlist
     int32_t* depth;          // [nd]
@@ -807,7 +807,10 @@ __global__ void __launch_bounds__(LD_THREADS, 1) k_levelise_dir(DirLevArgs a) {
             ++L;
             __syncthreads();  // everyone has read s_next before it is reset
         }
-        if (threadIdx.x == 0) a.depth[d] = L;
+        if (threadIdx.x == 0) {
+            a.depth[d] = L;
+            a.n0[d] = (int32_t)base;  // cells levelised
+        }
         __syncthreads();
     }
 }
@@ -1411,10 +1414,30 @@ cudaError_t ensure_seg(Levels& L, int nlev) {
     return cudaSuccess;
 }
 
-// Direction-parallel levelisation. Sets *nlev_out, or *overflow when a direction is deeper than the
-// per-direction tables (the classification counters are then spent: classify again before retrying).
+// Device memory for the level-major task list.
+cudaError_t alloc_merged(Levels& L) {
+    cudaError_t e = cudaSuccess;
+    if (!L.task) e = cudaMalloc(&L.task, sizeof(uint32_t) * L.task_cap);
+    if (e == cudaSuccess && !L.trec) e = cudaMalloc(&L.trec, sizeof(int4) * L.task_cap);
+    return e;
+}
+
+// Level tables on the host (the packing and the plain schedule walk them).
+cudaError_t read_level_tables(Levels& L, cudaStream_t st) {
+    const int nlev = L.n_levels, nd = L.nd;
+    L.h_lev_chunk.assign(nlev + 1, 0);
+    L.h_seg_off.assign((size_t)nlev * (nd + 1), 0);
+    cudaMemcpyAsync(L.h_lev_chunk.data(), L.lev_chunk, sizeof(int64_t) * (nlev + 1), cudaMemcpyDeviceToHost, st);
+    if (nlev > 0)
+        cudaMemcpyAsync(L.h_seg_off.data(), L.seg_off, sizeof(uint32_t) * L.h_seg_off.size(), cudaMemcpyDeviceToHost, st);
+    return cudaStreamSynchronize(st);
+}
+
+// Direction-parallel levelisation. Sets L.n_levels, L.depth and *done (cells levelised), or *overflow when a
+// direction is deeper than the per-direction tables (the classification counters are then spent: classify
+// again before retrying).
 cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om32, const double* om64, int dev_sms,
-                                  cudaStream_t st, int* nlev_out, bool* overflow) {
+                                  cudaStream_t st, int64_t* done, bool* overflow) {
     const int nd = L.nd, cap = L.dlev_cap;
     int32_t* dcnt = L.dlev;
     int32_t* dbase = dcnt + (int64_t)nd * cap;
@@ -1432,19 +1455,20 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
     k_levelise_dir<<<blocks, LD_THREADS, LD_SMEM, st>>>(a);
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;
-    std::vector<int32_t> h(nd + 1);
-    cudaMemcpyAsync(h.data(), depth, sizeof(int32_t) * (nd + 1), cudaMemcpyDeviceToHost, st);
+    std::vector<int32_t> h(2 * nd + 1);
+    cudaMemcpyAsync(h.data(), n0, sizeof(int32_t) * (2 * nd + 1), cudaMemcpyDeviceToHost, st);
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
-    *overflow = h[nd] != 0;
+    *overflow = h[2 * nd] != 0;
     if (*overflow) return cudaSuccess;
-    int nlev = 0;
-    for (int d = 0; d < nd; ++d) nlev = std::max(nlev, h[d]);
-    *nlev_out = nlev;
-    if (nlev == 0) {
-        cudaMemsetAsync(L.pad_off, 0, sizeof(uint32_t), st);
-        return cudaMemsetAsync(L.lev_chunk, 0, sizeof(int64_t), st);
+    *done = 0;
+    L.depth.assign(h.begin() + nd, h.begin() + 2 * nd);
+    L.n_levels = 0;
+    for (int d = 0; d < nd; ++d) {
+        *done += h[d];
+        L.n_levels = std::max(L.n_levels, L.depth[d]);
     }
+    if (L.n_levels == 0) return cudaSuccess;
     // the cells of each (direction, level) in cell order
     if (!L.lfill) {
         if ((e = cudaMalloc(&L.lfill, sizeof(int32_t) * (size_t)nd * cap))) return e;
@@ -1452,13 +1476,6 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
     if ((e = cudaMemsetAsync(L.lfill, 0, sizeof(int32_t) * (size_t)nd * cap, st))) return e;
     const int64_t tot = m.N * (int64_t)nd;
     if (tot > 0) k_order_levels<<<nblk(tot), 256, 0, st>>>(m.N, nd, cap, L.level, dbase, L.lfill, L.raw);
-    e = ensure_seg(L, nlev);
-    if (e != cudaSuccess) return e;
-    k_level_totals<<<nblk(nlev), 256, 0, st>>>(dcnt, depth, nd, cap, nlev, L.lvl_cnt);
-    k_level_starts<<<1, 1024, 0, st>>>(L.lvl_cnt, nlev, L.pad_off, L.lev_chunk);
-    k_seg_starts<<<nblk(nlev), 256, 0, st>>>(dcnt, depth, nd, cap, nlev, L.pad_off, L.seg_off);
-    k_gather_levels<<<nlev, 256, 0, st>>>(L.raw, dcnt, dbase, depth, m.N, nd, cap, L.cshift, L.pad_off, L.lvl_cnt,
-                                          L.seg_off, m.rowptr, L.info, L.task, L.trec);
     return cudaGetLastError();
 }
 
@@ -1499,6 +1516,7 @@ cudaError_t levelise_all(const DevMesh& m, Levels& L, const float4* om32, const 
     *nlev_out = nlev;
     if (*timed_out || nlev == 0) return cudaSuccess;
     e = ensure_seg(L, nlev);
+    if (e == cudaSuccess) e = alloc_merged(L);
     if (e != cudaSuccess) return e;
     k_sort_levels<<<nlev, 256, 2 * L.nd * sizeof(int), st>>>(L.raw, L.task, L.pad_off, L.lvl_cnt, L.nd, L.cshift,
                                                               L.seg_off, L.cmask, m.rowptr, L.info, L.trec);
@@ -1506,6 +1524,31 @@ cudaError_t levelise_all(const DevMesh& m, Levels& L, const float4* om32, const 
 }
 
 }  // namespace
+
+cudaError_t merge_levels(const DevMesh& m, Levels& L, cudaStream_t st) {
+    if (L.merged) return cudaSuccess;
+    const int nd = L.nd, cap = L.dlev_cap, nlev = L.n_levels;
+    const int32_t* dcnt = L.dlev;
+    const int32_t* dbase = dcnt + (int64_t)nd * cap;
+    const int32_t* depth = dbase + (int64_t)nd * cap + nd;
+    cudaError_t e = alloc_merged(L);
+    if (e != cudaSuccess) return e;
+    if (nlev == 0) {
+        cudaMemsetAsync(L.pad_off, 0, sizeof(uint32_t), st);
+        cudaMemsetAsync(L.lev_chunk, 0, sizeof(int64_t), st);
+    } else {
+        if ((e = ensure_seg(L, nlev))) return e;
+        k_level_totals<<<nblk(nlev), 256, 0, st>>>(dcnt, depth, nd, cap, nlev, L.lvl_cnt);
+        k_level_starts<<<1, 1024, 0, st>>>(L.lvl_cnt, nlev, L.pad_off, L.lev_chunk);
+        k_seg_starts<<<nblk(nlev), 256, 0, st>>>(dcnt, depth, nd, cap, nlev, L.pad_off, L.seg_off);
+        k_gather_levels<<<nlev, 256, 0, st>>>(L.raw, dcnt, dbase, depth, m.N, nd, cap, L.cshift, L.pad_off, L.lvl_cnt,
+                                              L.seg_off, m.rowptr, L.info, L.task, L.trec);
+        if ((e = cudaGetLastError())) return e;
+    }
+    e = read_level_tables(L, st);
+    L.merged = e == cudaSuccess;
+    return e;
+}
 
 cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const float4* om32_all,
                      const float4* om32lo_all, int dev_sms, GridBar* bar, int* err, long long budget,
@@ -1550,13 +1593,15 @@ cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const 
         }
     }
     cudaEventRecord(ev[1], st);
-    int nlev = 0;
-    bool done_by_dir = false;
+    const int64_t tot = N * (int64_t)nd;
+    int64_t done = 0;
+    L.merged = false;
+    L.by_dir = false;
     if (by_dir) {
         bool overflow = false;
-        e = levelise_by_direction(m, L, om32, om64, dev_sms, st, &nlev, &overflow);
+        e = levelise_by_direction(m, L, om32, om64, dev_sms, st, &done, &overflow);
         if (e != cudaSuccess) return e;
-        done_by_dir = !overflow;
+        L.by_dir = !overflow;
         if (overflow && L.transport > 0) {
             *msg = "direction-conserving transport: a direction is deeper than 65536 levels";
             L.valid = false;
@@ -1567,8 +1612,9 @@ cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const 
             if (e != cudaSuccess) return e;
         }
     }
-    if (!done_by_dir) {
+    if (!L.by_dir) {
         bool timed_out = false;
+        int nlev = 0;
         e = levelise_all(m, L, om32, om64, dev_sms, bar, err, budget, d_scratch, st, &nlev, &timed_out);
         if (e != cudaSuccess) return e;
         if (timed_out) {
@@ -1576,35 +1622,29 @@ cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const 
             L.valid = false;
             return cudaSuccess;
         }
+        L.n_levels = nlev;
+        std::vector<int32_t> cnt(nlev > 0 ? nlev : 1);
+        if (nlev > 0) cudaMemcpyAsync(cnt.data(), L.lvl_cnt, sizeof(int32_t) * nlev, cudaMemcpyDeviceToHost, st);
+        if ((e = read_level_tables(L, st))) return e;
+        L.merged = true;
+        for (int i = 0; i < nlev; ++i) done += cnt[i];
+        L.depth.assign(nd, 0);
+        for (int lv = 0; lv < nlev; ++lv)
+            for (int d = 0; d < nd; ++d) {
+                uint32_t a0 = L.h_seg_off[(size_t)lv * (nd + 1) + d], a1 = L.h_seg_off[(size_t)lv * (nd + 1) + d + 1];
+                if (a1 > a0) L.depth[d] = lv + 1;
+            }
     }
-    L.n_levels = nlev;
-    std::vector<int32_t> cnt(nlev > 0 ? nlev : 1);
-    if (nlev > 0) cudaMemcpyAsync(cnt.data(), L.lvl_cnt, sizeof(int32_t) * nlev, cudaMemcpyDeviceToHost, st);
-    L.h_lev_chunk.assign(nlev + 1, 0);
-    cudaMemcpyAsync(L.h_lev_chunk.data(), L.lev_chunk, sizeof(int64_t) * (nlev + 1), cudaMemcpyDeviceToHost, st);
-    L.h_seg_off.assign((size_t)nlev * (nd + 1), 0);
-    if (nlev > 0)
-        cudaMemcpyAsync(L.h_seg_off.data(), L.seg_off, sizeof(uint32_t) * L.h_seg_off.size(), cudaMemcpyDeviceToHost,
-                        st);
     cudaEventRecord(ev[2], st);
     e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return e;
-    int64_t done = 0;
-    for (int i = 0; i < nlev; ++i) done += cnt[i];
     L.n_tasks = done;
-    const int64_t tot = N * (int64_t)nd;
     if (done != tot) {
         *msg = "dependency graph is cyclic: " + std::to_string(tot - done) + " tasks never became ready";
         L.valid = false;
         L.n_levels = 0;
         return cudaSuccess;
     }
-    L.depth.assign(nd, 0);
-    for (int lv = 0; lv < nlev; ++lv)
-        for (int d = 0; d < nd; ++d) {
-            uint32_t a0 = L.h_seg_off[(size_t)lv * (nd + 1) + d], a1 = L.h_seg_off[(size_t)lv * (nd + 1) + d + 1];
-            if (a1 > a0) L.depth[d] = lv + 1;
-        }
     float ms1 = 0, ms2 = 0;
     cudaEventElapsedTime(&ms1, ev[0], ev[1]);
     cudaEventElapsedTime(&ms2, ev[1], ev[2]);

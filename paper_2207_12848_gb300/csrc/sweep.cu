@@ -62,26 +62,6 @@ __device__ __forceinline__ void exp_update(double fin, double q, double ktv, dou
         out = mean = (q + fin) / ktv;
     }
 }
-// The same law in the packed kernel, where every lane of a packet evaluates it (the head lanes keep the
-// result): one expf and two fast reciprocals, selects instead of branches. The mean factor
-// f = (1 - exp(-tau)) / tau is taken from its Taylor series sum_k (-tau)^k / (k+1)! (seven terms,
-// truncation below 2e-9) where 1 - exp(-tau) would cancel (tau < 1/4), and directly above.
-__device__ __forceinline__ void exp_update_lanes(float fin, float q, float ktv, float P, float& out, float& mean) {
-    const float rP = __fdividef(1.f, P), rK = __fdividef(1.f, ktv);
-    const float tau = ktv * rP;
-    const float e = expf(-tau);
-    const float s = -tau;
-    float ft = fmaf(s, 1.f / 5040.f, 1.f / 720.f);
-    ft = fmaf(s, ft, 1.f / 120.f);
-    ft = fmaf(s, ft, 1.f / 24.f);
-    ft = fmaf(s, ft, 1.f / 6.f);
-    ft = fmaf(s, ft, 0.5f);
-    ft = fmaf(s, ft, 1.f);
-    const float f = tau < 0.25f ? ft : (1.f - e) * P * rK;
-    const float stay = (q + fin) * rK;  // P = 0: no outflow
-    out = P > 0.f ? fmaf(e, fin, q) * rP : stay;
-    mean = P > 0.f ? fin * rP * f : stay;
-}
 // out of line in the mesh-row kernels, whose common path stays short
 __device__ __noinline__ void exp_law(float fin, float q, float ktv, float P, float& out, float& mean) {
     exp_update(fin, q, ktv, P, out, mean);
