@@ -502,11 +502,6 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
     auto enqueue = [&](int t, cudaEvent_t* ev) -> cudaError_t {
         cudaError_t e;
         const int cur = cur_of(t);
-        if (scat) {  // scattering source from the previous J (Alg. 1)
-            if ((e = launch_prep_material(N, G, c->mesh.vol, c->ka, c->ks, c->em, c->Jold,
-                                          prec == 32 ? c->cm32 : nullptr, prec == 64 ? c->cm64 : nullptr, gs)))
-                return e;
-        }
         if ((e = cudaMemsetAsync(c->bar, 0, sizeof(GridBar), gs))) return e;
         if ((e = cudaMemsetAsync(c->derr, 0, sizeof(int), gs))) return e;
         if ((e = cudaEventRecordWithFlags(ev[0], gs, cudaEventRecordExternal))) return e;
@@ -523,14 +518,12 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
         }
         if (e) return e;
         if ((e = cudaEventRecordWithFlags(ev[1], gs, cudaEventRecordExternal))) return e;
-        if (scat) {
-            if ((e = launch_tally(prec, o.law ? c->Imean : b.I[cur], N, G, D, 0, c->w64, c->wsum, c->mesh.vol, c->ka,
-                                  c->em, c->J,
-                                  c->Gam, c->partial, nblk, gs)))
-                return e;
+        if (scat) {  // J, its change and the next sweep's source (Alg. 1)
             unsigned long long* ds = c->dmax + (fused ? 1 : 0);
             if ((e = cudaMemsetAsync(ds, 0, sizeof(unsigned long long), gs))) return e;
-            if ((e = launch_scat_residual(NG, c->J, c->Jold, ds, gs))) return e;
+            if ((e = launch_scat_update(prec, o.law ? c->Imean : b.I[cur], N, G, D, c->w64, c->mesh.vol, c->ks, c->em,
+                                        c->Jold, c->cm32, c->cm64, ds, gs)))
+                return e;
             if (fused && (e = cudaMemcpyAsync(&hp->dmax_scat, ds, sizeof(unsigned long long), cudaMemcpyDeviceToHost,
                                               gs)))
                 return e;
@@ -563,7 +556,7 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
     cudaStreamWaitEvent(gs, fork, 0);
     cudaEventDestroy(fork);
     *done = true;
-    const int per_iter = (pbc ? 3 : 1) + (scat ? 3 : 0);  // kernels per iteration
+    const int per_iter = (pbc ? 3 : 1) + (scat ? 1 : 0);  // kernels per iteration
     for (int it = 0;; ++it) {
         const int t = it % period;
         CK(cudaGraphLaunch(gset.ex[t], gs), "graph launch");
@@ -1366,12 +1359,10 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     // Sec. 2.7's fused loops: one source-iteration sweep per periodic iteration, J carried over
     const bool fused = o.fused_loops && has_pbc && c->has_scat;
     if (o.use_graph && !plain && !o.debug_stall && (has_pbc != c->has_scat || fused)) {
-        // what stays fixed over the iterations: the source without scattering, J_old before Alg. 1
-        if (has_pbc && !fused)
-            CKL(launch_prep_material(N, G, c->mesh.vol, c->ka, c->ks, c->em, nullptr, prec == 32 ? c->cm32 : nullptr,
-                                    prec == 64 ? c->cm64 : nullptr, c->st), "prep");
-        else
-            CK(cudaMemsetAsync(c->Jold, 0, sizeof(double) * NG, c->st), "init");
+        // the source of the first sweep (no scattering yet), J_old before Alg. 1
+        CKL(launch_prep_material(N, G, c->mesh.vol, c->ka, c->ks, c->em, nullptr, prec == 32 ? c->cm32 : nullptr,
+                                prec == 64 ? c->cm64 : nullptr, c->st), "prep");
+        if (c->has_scat) CK(cudaMemsetAsync(c->Jold, 0, sizeof(double) * NG, c->st), "init");
         LoopState ls;
         ls.cur = cur;
         ls.prev = prev;
@@ -1396,11 +1387,14 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     }
     S.graph_used = graphed ? 1 : 0;
     for (; !graphed;) {
-        if (!fused || it_pbc == 0) CK(cudaMemsetAsync(c->Jold, 0, sizeof(double) * NG, c->st), "init");
+        // the source iteration starts from J = 0; each sweep's update leaves the next sweep's source
+        if (it_pbc == 0 || (c->has_scat && !fused)) {
+            if (c->has_scat) CK(cudaMemsetAsync(c->Jold, 0, sizeof(double) * NG, c->st), "init");
+            CKL(launch_prep_material(N, G, c->mesh.vol, c->ka, c->ks, c->em, nullptr, prec == 32 ? c->cm32 : nullptr,
+                                    prec == 64 ? c->cm64 : nullptr, c->st), "prep");
+        }
         int it_scat = 0;
         for (;;) {
-            CKL(launch_prep_material(N, G, c->mesh.vol, c->ka, c->ks, c->em, c->has_scat ? c->Jold : nullptr,
-                                    prec == 32 ? c->cm32 : nullptr, prec == 64 ? c->cm64 : nullptr, c->st), "prep");
             const int parity = !b.sign[cur];
             SweepArgs a = make_args(c, c->lev, prec, cm, b.I[cur], has_pbc ? b.I[prev] : nullptr, G, parity, 0, 0, &o);
             a.debug_stall = o.debug_stall && n_sweeps == 0;
@@ -1413,10 +1407,10 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
             // without scattering nothing inside the iteration needs J: the final tally below computes it
             if (!c->has_scat) break;
             cudaEventRecord(u0, c->st);
-            CKL(launch_tally(prec, o.law ? c->Imean : b.I[cur], N, G, D, 0, c->w64, c->wsum, c->mesh.vol, c->ka,
-                            c->em, c->J, c->Gam, c->partial, nblk, c->st), "tally");
             CK(cudaMemsetAsync(c->dmax, 0, sizeof(unsigned long long), c->st), "init");
-            CKL(launch_scat_residual(NG, c->J, c->Jold, c->dmax, c->st), "scattering residual");
+            CKL(launch_scat_update(prec, o.law ? c->Imean : b.I[cur], N, G, D, c->w64, c->mesh.vol, c->ks, c->em, c->Jold,
+                                  c->cm32, c->cm64, c->dmax, c->st),
+               "scattering update");
             cudaEventRecord(u1, c->st);
             res_scat = read_max(c);
             float tt = 0;

@@ -549,8 +549,9 @@ struct DcTabs {
 cudaError_t launch_boundary_tally(int precision, const DevMesh& m, const void* I, int G, int nd, int d0,
                                   const double* om64, const double* w64, const double* bc, double* partial,
                                   int nblk, cudaStream_t st, const DcTabs* dc = nullptr);
-cudaError_t launch_scat_residual(int64_t NG, const double* J, double* Jold, unsigned long long* d_max,
-                                 cudaStream_t st);
+cudaError_t launch_scat_update(int precision, const void* I, int64_t N, int G, int nd, const double* w64, const double* vol,
+                               const double* ks, const double* em, double* Jold, float2* cm32, double2* cm64,
+                               unsigned long long* d_max, cudaStream_t st);
 // FP64 periodic-inflow weights of a solve (periodic sides of the periodic cells x directions)
 struct PeriodicTable {
     int32_t* off = nullptr;   // [n_pcells+1] first periodic side of each periodic cell, then scratch counts
