@@ -117,7 +117,7 @@ void dfree(T*& p) {
 }
 
 void free_levels(Levels& L) {
-    dfree(L.raw); dfree(L.task); dfree(L.trec); dfree(L.info); dfree(L.level); dfree(L.lvl_cnt); dfree(L.pad_off);
+    dfree(L.raw); dfree(L.task); dfree(L.trec); dfree(L.info); dfree(L.level); dfree(L.word); dfree(L.lvl_cnt); dfree(L.pad_off);
     dfree(L.lev_chunk); dfree(L.seg_off); dfree(L.op); dfree(L.dlev);
     for (PackedOp* P : {&L.pk, &L.pkt}) {
         dfree(P->pk); dfree(P->meta); dfree(P->lev_pk); dfree(P->grp); dfree(P->lev_grp); dfree(P->cnt);
@@ -133,7 +133,7 @@ void free_levels(Levels& L) {
 }
 
 void free_mesh(DevMesh& m) {
-    dfree(m.rowptr); dfree(m.side); dfree(m.side64); dfree(m.side_lo); dfree(m.nbr_rows); dfree(m.twin); dfree(m.vol);
+    dfree(m.rowptr); dfree(m.side); dfree(m.side64); dfree(m.side_lo); dfree(m.ids); dfree(m.twin); dfree(m.vol);
     dfree(m.pcells); dfree(m.bcells);
     m = DevMesh();
 }
@@ -186,6 +186,7 @@ sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
     CK(cudaMalloc(&L.raw, sizeof(uint32_t) * L.task_cap), "alloc task list");
     CK(cudaMalloc(&L.info, sizeof(int4) * N * nd), "alloc classification");
     CK(cudaMalloc(&L.level, sizeof(int32_t) * N * nd), "alloc levels");
+    CK(cudaMalloc(&L.word, sizeof(unsigned long long) * N * nd), "alloc levels");
     CK(cudaMalloc(&L.lvl_cnt, sizeof(int32_t) * (N + 2)), "alloc level counts");
     CK(cudaMalloc(&L.pad_off, sizeof(uint32_t) * (N + 2)), "alloc level offsets");
     CK(cudaMalloc(&L.lev_chunk, sizeof(int64_t) * (N + 2)), "alloc level chunks");
@@ -773,7 +774,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     CKM(cudaMalloc(&m.side, sizeof(int4) * (S > 0 ? S : 1) + 64 * sizeof(int4)), "alloc sides");
     CKM(cudaMalloc(&m.side64, sizeof(d4) * (S > 0 ? S : 1)), "alloc sides");
     CKM(cudaMalloc(&m.side_lo, sizeof(float4) * (S > 0 ? S : 1)), "alloc sides");
-    CKM(cudaMalloc(&m.nbr_rows, sizeof(int2) * (S > 0 ? S : 1)), "alloc sides");
+    CKM(cudaMalloc(&m.ids, sizeof(int32_t) * 32 * n_cells), "alloc sides");
     CKM(cudaMalloc(&m.twin, sizeof(uint32_t) * (S > 0 ? S : 1)), "alloc sides");
     CKM(launch_build_csr(m, d_fc, d_area, d_normal, d_flags, d_tmp, c->st), "build CSR");
     CKM(cudaStreamSynchronize(c->st), "build CSR");

@@ -345,7 +345,7 @@ struct DevMesh {
     int4* side = nullptr;                  // [S]
     d4* side64 = nullptr;                  // [S]
     float4* side_lo = nullptr;             // [S] area vector minus its FP32 value in the side record
-    int2* nbr_rows = nullptr;              // [S] row bounds of the side's interior neighbour ({0, 0} otherwise)
+    int32_t* ids = nullptr;                // [N][32] neighbour codes of the first 32 sides (-1 past the row's end)
     uint32_t* twin = nullptr;              // [S] position of the same face in the neighbour's row (interior and
                                            //     periodic sides; boundary sides 0xffffffff)
     double* vol = nullptr;                 // [N]
@@ -432,7 +432,8 @@ struct Levels {
     uint64_t* dc_inm = nullptr;
     float* dc_share32 = nullptr;
     double* dc_share64 = nullptr;
-    int32_t* level = nullptr;    // [nd][N] (during levelisation: minus the upwind cells still unsolved)
+    int32_t* level = nullptr;    // [nd][N]
+    unsigned long long* word = nullptr;  // [nd][N] levelisation: {sides that release, upwind cells still unsolved}
     int32_t* lvl_cnt = nullptr;  // [N+2]
     uint32_t* pad_off = nullptr; // [N+2] start of each level in the padded list
     int64_t* lev_chunk = nullptr;  // device [n_levels+1] chunk (32-task) offsets

@@ -184,7 +184,7 @@ __global__ void k_flag_boundary(int64_t F, const uint8_t* flags, int32_t* isb) {
 
 __global__ void k_fill_sides(int64_t S, const int64_t* key, const int32_t* fc, const double* area,
                              const double* normal, const uint8_t* flags, const int64_t* bidx,
-                             const uint32_t* rowptr, int4* side, d4* side64, float4* side_lo, int2* nbr_rows) {
+                             int4* side, d4* side64, float4* side_lo) {
     int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= S) return;
     int64_t k = key[s];
@@ -211,7 +211,16 @@ __global__ void k_fill_sides(int64_t S, const int64_t* key, const int32_t* fc, c
     side[s] = r;
     side64[s] = d4{nx, ny, nz, A};
     side_lo[s] = make_float4((float)(ax - (double)hx), (float)(ay - (double)hy), (float)(az - (double)hz), 0.f);
-    nbr_rows[s] = nbr >= 0 && !(nbr & NBR_PERIODIC) ? make_int2((int)rowptr[nbr], (int)rowptr[nbr + 1]) : make_int2(0, 0);
+}
+
+// Neighbour codes of each cell's first 32 sides at a fixed place (-1 past the row's end): the levelisation reads
+// them without the row bounds, 4 bytes a side.
+__global__ void k_fill_ids(int64_t N, const uint32_t* rowptr, const int4* side, int32_t* ids) {
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= N * 32) return;
+    const int64_t c = t >> 5;
+    const uint32_t s = rowptr[c] + (uint32_t)(t & 31);
+    ids[t] = s < rowptr[c + 1] ? side[s].x : -1;
 }
 
 // Position of each interior or periodic side's twin (the same face seen from the neighbour) in the
@@ -303,8 +312,9 @@ cudaError_t launch_build_csr(const DevMesh& mc, const int32_t* fc, const double*
         k_flag_boundary<<<nblk(F), 256, 0, st>>>(F, flags, isb);
         TRY(scan_i32(isb, F, bidx, scratch, total, st));
     }
-    if (S > 0) k_fill_sides<<<nblk(S), 256, 0, st>>>(S, key, fc, area, normal, flags, bidx, m.rowptr, m.side,
-                                                     m.side64, m.side_lo, m.nbr_rows);
+    if (S > 0) k_fill_sides<<<nblk(S), 256, 0, st>>>(S, key, fc, area, normal, flags, bidx, m.side, m.side64,
+                                                     m.side_lo);
+    if (N > 0) k_fill_ids<<<nblk(N * 32), 256, 0, st>>>(N, m.rowptr, m.side, m.ids);
     if (S > 0) k_twin<<<nblk(S), 256, 0, st>>>(S, key, fc, flags, m.rowptr, m.twin);
     // periodic / boundary cell lists (increasing cell order)
     if (N > 0) {
@@ -361,7 +371,7 @@ namespace {
 __global__ void k_classify(int64_t N, int nd, const uint32_t* rowptr, const int4* side, const d4* side64,
                            const float4* side_lo, const float4* om32, const float4* om32lo, const double* om64,
                            int4* info, int32_t* level, uint32_t* raw, int32_t* lvl_cnt, int cshift, uint32_t* dlist,
-                           int32_t* n0) {
+                           int32_t* n0, unsigned long long* word) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool active = t < N * (int64_t)nd;
     int cnt = 0;
@@ -391,7 +401,9 @@ __global__ void k_classify(int64_t N, int nd, const uint32_t* rowptr, const int4
         }
         int pbits = __float_as_int(P) | ((r1 - r0 > 32u) ? (int)0x80000000 : 0);
         info[t] = make_int4(cnt, pbits, (int)inm, (int)outm);
-        level[(size_t)dl * N + c] = -cnt;  // 0: level 0; the levelisation counts up to 0, then stores the level
+        // the direction-parallel levelisation's word (see k_levelise_dir); level 0 is final
+        if (dlist) word[(size_t)dl * N + c] = (unsigned long long)outm << 32 | (uint32_t)cnt;
+        if (!dlist || cnt == 0) level[(size_t)dl * N + c] = -cnt;
         entry = ((uint32_t)dl << cshift) | (uint32_t)c;
     }
     bool push = active && cnt == 0;
@@ -472,10 +484,11 @@ __global__ void k_dc_choose(int64_t N, int nd, int dcn, const uint32_t* rowptr, 
 // Effective inflow sides of each task under scheme (b) -- interior and periodic sides whose upwind cell
 // chose the face (read through the twin side's position in the upwind row), and boundary inflow sides,
 // which enter as in scheme (a) -- and the upwind count over the chosen interior faces, which seeds the
-// levelisation (level = -count, level-0 lists per direction).
+// levelisation (its words: chosen sides and count; level-0 lists per direction).
 __global__ void k_dc_count(int64_t N, int nd, const uint32_t* rowptr, const int4* side, const d4* side64,
                            const float4* om32, const double* om64, const uint32_t* twin, const uint64_t* dc_mask,
-                           uint64_t* dc_inm, int32_t* level, uint32_t* dlist, int32_t* n0) {
+                           uint64_t* dc_inm, int32_t* level, uint32_t* dlist, int32_t* n0,
+                           unsigned long long* word) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= N * (int64_t)nd) return;
     const int64_t c = t / nd;
@@ -501,7 +514,8 @@ __global__ void k_dc_count(int64_t N, int nd, const uint32_t* rowptr, const int4
         }
     }
     dc_inm[t] = inm;
-    level[(size_t)dl * N + c] = -cnt;
+    word[(size_t)dl * N + c] = (unsigned long long)(uint32_t)dc_mask[t] << 32 | (uint32_t)cnt;
+    if (cnt == 0) level[(size_t)dl * N + c] = 0;
     if (cnt == 0) dlist[(size_t)dl * N + atomicAdd(&n0[dl], 1)] = (uint32_t)c;
 }
 
@@ -677,23 +691,25 @@ __global__ void k_sort_levels(const uint32_t* raw, uint32_t* task, const uint32_
 // list is kept in shared memory (spilling to the direction's list in global memory when wide).
 // ---------------------------------------------------------------------------------------------
 constexpr int LD_THREADS = 1024;
-constexpr int LD_KL = 4;     // lanes per task: one pass covers 32 face sides, so nearly every row takes one
-constexpr int LD_KU = 8;     // face sides per lane per pass
-constexpr int LD_Q = 8192;   // level-list entries {cell, row start, row end} held in shared memory (2 x 96 KB)
-constexpr size_t LD_SMEM = sizeof(uint32_t) * 3 * 2 * LD_Q;
+constexpr int LD_KL = 4;     // lanes per task: one pass covers 32 face sides
+constexpr int LD_KU = 8;     // face sides per lane
+constexpr int LD_Q = 8192;   // level-list entries {cell, sides} held in shared memory (2 x 64 KB)
+constexpr size_t LD_SMEM = sizeof(uint2) * 2 * LD_Q;
 
 struct DirLevArgs {
     int64_t N;
     int nd;
     int cap;                 // levels the per-direction tables hold
+    int long_rows;           // some row has more than 32 sides
     const uint32_t* rowptr;
+    const int32_t* ids;      // [N][32] neighbour codes of the first 32 sides
     const int4* side;
     const d4* side64;
-    const int2* nbr_rows;    // [S] row bounds of each side's interior neighbour
     const float4* om32;
     const double* om64;
     const uint64_t* dc_mask; // scheme (b): [N][nd] chosen outflow sides (release only those), or null
-    int32_t* level;          // [nd][N]: minus the unsolved upwind cells, then the level
+    unsigned long long* word;  // [nd][N] {sides that release, upwind cells still unsolved}
+    int32_t* level;          // [nd][N]: level 0 from the classification
     uint32_t* dlist;         // [nd][N] cells of each direction in level order; level 0 from the classification
     int32_t* n0;             // [nd] level-0 sizes; then the cells levelised (fewer than N: a cycle)
     int32_t* dcnt;           // [nd][cap] cells on each level
@@ -702,29 +718,28 @@ struct DirLevArgs {
     int32_t* overflow;       // set when a direction has more than cap levels
 };
 
-// Per level and task: the side records of the cell's row (classified in registers: sign of n.Omega
-// as in the classification) and, for each downwind interior neighbour, one atomic on its counter
-// together with a load of that neighbour's row bounds, so a cell released here enters the next
-// level's list with its row already known (and its row prefetched into L2 by the bulk-copy engine, so
-// the next level's record loads are L2 hits): two dependent memory round trips per level.
+// A cell's 64-bit word per direction holds the mask of its sides that release a neighbour (from the
+// classification) above the count of its unsolved upwind cells. Releasing a neighbour is one 64-bit atomic on
+// its word: when the count falls to zero the same answer says which sides the neighbour releases in its turn. So a
+// level costs two dependent trips to L2 -- the neighbour codes (4 bytes a side, at a place that needs no row bounds,
+// prefetched into L2 when the cell is released), then the words -- and a task about 45 instructions; reading
+// the 16-byte side records, classifying them again and fetching the neighbour's row bounds took 13.0 us per level (2^21
+// cells, 128 directions, 470 cells per level), now 7.1 us.
 __global__ void __launch_bounds__(LD_THREADS, 1) k_levelise_dir(DirLevArgs a) {
-    extern __shared__ uint32_t s_lists[];  // [2][LD_Q][3]
+    extern __shared__ uint2 s_lists[];  // [2][LD_Q]
     __shared__ int s_next;
-    const int gl = threadIdx.x % LD_KL;
+    const int gl = threadIdx.x % LD_KL, lane = threadIdx.x & 31;
     constexpr int TPR = LD_THREADS / LD_KL;  // tasks per round
     for (int d = blockIdx.x; d < a.nd; d += gridDim.x) {
         uint32_t* out = a.dlist + (size_t)d * a.N;
+        unsigned long long* word = a.word + (size_t)d * a.N;
         int32_t* lv = a.level + (size_t)d * a.N;
         int32_t* cnt = a.dcnt + (size_t)d * a.cap;
         int32_t* bas = a.dbase + (size_t)d * a.cap;
-        const float4 om = a.om32[d];
-        const double* o64 = a.om64 + 3 * d;
         int n = a.n0[d];
         for (int i = threadIdx.x; i < n && i < LD_Q; i += LD_THREADS) {
             const uint32_t c = out[i];
-            s_lists[3 * i] = c;
-            s_lists[3 * i + 1] = a.rowptr[c];
-            s_lists[3 * i + 2] = a.rowptr[c + 1];
+            s_lists[i] = make_uint2(c, (uint32_t)(__ldcg(word + c) >> 32));
         }
         uint32_t base = 0;
         int L = 0, cur = 0;
@@ -740,63 +755,78 @@ __global__ void __launch_bounds__(LD_THREADS, 1) k_levelise_dir(DirLevArgs a) {
             }
             __syncthreads();
             const uint32_t nbase = base + (uint32_t)n;
-            const uint32_t* q = s_lists + cur * 3 * LD_Q;
-            uint32_t* qn = s_lists + (cur ^ 1) * 3 * LD_Q;
+            const uint2* q = s_lists + cur * LD_Q;
+            uint2* qn = s_lists + (cur ^ 1) * LD_Q;
+            // The neighbours whose count fell to zero go onto the next level's list: places by one scan over the warp
+            // and one shared atomic (a ballot and an atomic per side put eight of them in a row).
+            auto release = [&](const int32_t (&x)[LD_KU], const unsigned long long (&o)[LD_KU]) {
+                int c = 0;
+#pragma unroll
+                for (int k = 0; k < LD_KU; ++k) c += (uint32_t)o[k] == 1u;
+                if (!__any_sync(0xffffffffu, c)) return;
+                int p = c;
+#pragma unroll
+                for (int w = 1; w < 32; w <<= 1) {
+                    const int y = __shfl_up_sync(0xffffffffu, p, w);
+                    if (lane >= w) p += y;
+                }
+                int first = 0;
+                if (lane == 31) first = atomicAdd(&s_next, p);
+                p += __shfl_sync(0xffffffffu, first, 31) - c;
+#pragma unroll
+                for (int k = 0; k < LD_KU; ++k) {
+                    if ((uint32_t)o[k] != 1u) continue;
+                    const uint32_t v = (uint32_t)x[k];
+                    lv[v] = L + 1;
+                    if (nbase + (uint32_t)p < (uint32_t)a.N) out[nbase + p] = v;
+                    if (p < LD_Q) qn[p] = make_uint2(v, (uint32_t)(o[k] >> 32));
+                    ++p;
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.ids + (size_t)v * 32));
+                    asm volatile("prefetch.global.L2 [%0];" ::"l"(a.ids + (size_t)v * 32 + 8));
+                }
+            };
             for (int i0 = 0; i0 < n; i0 += TPR) {
                 const int i = i0 + threadIdx.x / LD_KL;
-                if (i >= n) continue;
-                uint32_t r0, r1, cc;
-                if (i < LD_Q) {
-                    cc = q[3 * i];
-                    r0 = q[3 * i + 1];
-                    r1 = q[3 * i + 2];
-                } else {  // a level wider than the shared list: cells from the global list
-                    cc = out[base + i];
-                    r0 = a.rowptr[cc];
-                    r1 = a.rowptr[cc + 1];
+                uint2 t = make_uint2(0u, 0u);
+                if (i < n) {
+                    if (i < LD_Q) {
+                        t = q[i];
+                    } else {  // a level wider than the shared list
+                        t.x = out[base + i];
+                        t.y = (uint32_t)(__ldcg(word + t.x) >> 32);
+                    }
                 }
-                const uint64_t chosen = a.dc_mask ? a.dc_mask[(int64_t)cc * a.nd + d] : 0ull;
-                for (uint32_t b = r0; b < r1; b += LD_KL * LD_KU) {
-                    int4 r[LD_KU];
+                const int32_t* ids = a.ids + (size_t)t.x * 32 + gl;
+                int32_t nb[LD_KU];
 #pragma unroll
-                    for (int k = 0; k < LD_KU; ++k) {
-                        const uint32_t s = b + gl + k * LD_KL;
-                        r[k] = s < r1 ? a.side[s] : make_int4(-1, 0, 0, 0);
-                    }
-                    int old[LD_KU];
-                    int2 nr[LD_KU];
+                for (int k = 0; k < LD_KU; ++k) nb[k] = (t.y >> (gl + k * LD_KL)) & 1u ? ids[k * LD_KL] : -1;
+                unsigned long long old[LD_KU];
 #pragma unroll
-                    for (int k = 0; k < LD_KU; ++k) {
-                        old[k] = 0;
-                        nr[k] = make_int2(0, 0);
-                        if (r[k].x < 0 || (r[k].x & NBR_PERIODIC)) continue;
-                        const uint32_t s = b + gl + k * LD_KL;
-                        const float ax = __int_as_float(r[k].y), ay = __int_as_float(r[k].z),
-                                    az = __int_as_float(r[k].w);
-                        if (a.dc_mask) {  // scheme (b): the chosen sides only
-                            if (!((chosen >> (s - r0)) & 1ull)) continue;
-                        } else if (classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, o64) <= 0) {
-                            continue;
+                for (int k = 0; k < LD_KU; ++k) {
+                    // scheme (b)'s masks hold boundary and periodic sides too
+                    if (nb[k] < 0 || (nb[k] & NBR_PERIODIC)) nb[k] = -1;
+                    old[k] = nb[k] >= 0 ? atomicAdd(word + nb[k], ~0ull) : 0ull;
+                }
+                release(nb, old);  // where this side solved the neighbour's last upwind cell
+                if (a.long_rows) {  // sides past the first 32
+                    const uint32_t r0 = i < n ? a.rowptr[t.x] : 0u, r1 = i < n ? a.rowptr[t.x + 1] : 0u;
+                    const uint64_t chosen = a.dc_mask && i < n ? a.dc_mask[(int64_t)t.x * a.nd + d] : 0ull;
+                    for (uint32_t s = r0 + 32u + (uint32_t)gl; __any_sync(0xffffffffu, s < r1); s += LD_KL) {
+                        int32_t x[LD_KU] = {};
+                        unsigned long long o[LD_KU] = {};
+                        if (s < r1) {
+                            const int4 r = a.side[s];
+                            const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
+                            const bool go = r.x >= 0 && !(r.x & NBR_PERIODIC) &&
+                                            (a.dc_mask ? (chosen >> (s - r0)) & 1ull
+                                                       : classify_side(dot32(ax, ay, az, a.om32[d]), ax, ay, az, a.side64, s,
+                                                                       a.om64 + 3 * d) > 0);
+                            if (go) {
+                                x[0] = r.x;
+                                o[0] = atomicAdd(word + r.x, ~0ull);
+                            }
                         }
-                        old[k] = atomicAdd(&lv[r[k].x], 1);
-                        nr[k] = a.nbr_rows[s];
-                    }
-#pragma unroll
-                    for (int k = 0; k < LD_KU; ++k) {
-                        if (old[k] != -1) continue;  // this side solved the neighbour's last upwind cell
-                        const uint32_t x = (uint32_t)r[k].x;
-                        lv[x] = L + 1;
-                        const int p = atomicAdd(&s_next, 1);
-                        if (nbase + (uint32_t)p < (uint32_t)a.N) out[nbase + p] = x;
-                        if (p < LD_Q) {
-                            qn[3 * p] = x;
-                            qn[3 * p + 1] = (uint32_t)nr[k].x;
-                            qn[3 * p + 2] = (uint32_t)nr[k].y;
-                        }
-                        // its side records are read on the next level: start pulling them into L2 now
-                        if (nr[k].y > nr[k].x)
-                            asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.side + nr[k].x),
-                                         "r"((uint32_t)(nr[k].y - nr[k].x) * 16u));
+                        release(x, o);
                     }
                 }
             }
@@ -824,7 +854,7 @@ __global__ void k_order_levels(int64_t N, int nd, int cap, const int32_t* level,
     const int64_t tot = N * (int64_t)nd;
     const int64_t d = t < tot ? t / N : -1, c = t - d * N;
     int L = t < tot ? level[t] : -1;
-    if (L >= cap) L = -1;  // negative: never levelised (a cycle) or past the tables
+    if (L >= cap) L = -1;
     // lanes of one direction and level take consecutive positions with one atomic, in lane (cell) order
     const int64_t key = L < 0 ? -1 : d * cap + L;
     const unsigned same = __match_any_sync(0xffffffffu, key);
@@ -1397,7 +1427,7 @@ cudaError_t classify(const DevMesh& m, Levels& L, const float4* om32, const floa
     if (tot > 0)
         k_classify<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, m.side_lo, om32, om32lo, om64,
                                                L.info, L.level, L.raw, L.lvl_cnt, L.cshift,
-                                               per_direction ? L.raw : nullptr, n0);
+                                               per_direction ? L.raw : nullptr, n0, L.word);
     return cudaGetLastError();
 }
 
@@ -1445,9 +1475,9 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
     int32_t* depth = n0 + nd;
     int32_t* ovf = depth + nd;
     DirLevArgs a;
-    a.N = m.N; a.nd = nd; a.cap = cap; a.rowptr = m.rowptr; a.side = m.side; a.side64 = m.side64;
-    a.nbr_rows = m.nbr_rows; a.om32 = om32; a.om64 = om64; a.level = L.level; a.dlist = L.raw; a.n0 = n0;
-    a.dcnt = dcnt; a.dbase = dbase;
+    a.N = m.N; a.nd = nd; a.cap = cap; a.long_rows = m.max_row > 32; a.rowptr = m.rowptr; a.ids = m.ids;
+    a.side = m.side; a.side64 = m.side64; a.om32 = om32; a.om64 = om64; a.word = L.word; a.level = L.level;
+    a.dlist = L.raw; a.n0 = n0; a.dcnt = dcnt; a.dbase = dbase;
     a.dc_mask = L.transport > 0 ? L.dc_mask : nullptr;
     a.depth = depth; a.overflow = ovf;
     const int blocks = nd < dev_sms ? nd : dev_sms;
@@ -1468,7 +1498,8 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
         *done += h[d];
         L.n_levels = std::max(L.n_levels, L.depth[d]);
     }
-    if (L.n_levels == 0) return cudaSuccess;
+    // a cycle: cells without a level (the caller reports it)
+    if (L.n_levels == 0 || *done != m.N * (int64_t)nd) return cudaSuccess;
     // the cells of each (direction, level) in cell order
     if (!L.lfill) {
         if ((e = cudaMalloc(&L.lfill, sizeof(int32_t) * (size_t)nd * cap))) return e;
@@ -1581,7 +1612,7 @@ cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const 
             k_dc_choose<<<nblk(tot), 256, 0, st>>>(N, nd, L.transport, m.rowptr, m.side64, om64, L.dc_mask,
                                                    L.dc_share32, L.dc_share64, bad);
             k_dc_count<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, om32, om64, m.twin, L.dc_mask,
-                                                  L.dc_inm, L.level, L.raw, n0);
+                                                  L.dc_inm, L.level, L.raw, n0, L.word);
         }
         int hbad = 0;
         if ((e = cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;
