@@ -77,6 +77,7 @@ struct sweep_ctx {
     int tuned[2][9][3][4] = {};  // [precision][groups][operator form OPF_*] -> schedule, threads, lanes, blocks/SM
     int64_t launches = 0;  // kernels launched by this context
     PeriodicTable ptab;          // periodic-inflow weights, rebuilt at the start of each periodic solve
+    MemPool pool;                // device memory given up by the buffers above and kept for the next ones
     cudaStream_t gst = nullptr;  // capture/replay stream of the iteration graphs
     void* hpin = nullptr;        // pinned host words the iteration graphs write
 };
@@ -112,7 +113,7 @@ sweep_status bad(sweep_ctx* c, const std::string& m) {
 
 template <typename T>
 void dfree(T*& p) {
-    if (p) cudaFree((void*)p);
+    if (p) dev_free((void*)p);
     p = nullptr;
 }
 
@@ -183,15 +184,15 @@ sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
     L.cmask = (bits == 32) ? 0u : ((1u << L.cshift) - 1u);
     if ((uint64_t)N > (uint64_t)L.cmask + 1ull) return bad(c, "n_cells too large for the number of directions");
     L.task_cap = N * (int64_t)nd + 32 * (N + 2);
-    CK(cudaMalloc(&L.raw, sizeof(uint32_t) * L.task_cap), "alloc task list");
-    CK(cudaMalloc(&L.info, sizeof(int4) * N * nd), "alloc classification");
-    CK(cudaMalloc(&L.level, sizeof(int32_t) * N * nd), "alloc levels");
-    CK(cudaMalloc(&L.word, sizeof(unsigned long long) * N * nd), "alloc levels");
-    CK(cudaMalloc(&L.lvl_cnt, sizeof(int32_t) * (N + 2)), "alloc level counts");
-    CK(cudaMalloc(&L.pad_off, sizeof(uint32_t) * (N + 2)), "alloc level offsets");
-    CK(cudaMalloc(&L.lev_chunk, sizeof(int64_t) * (N + 2)), "alloc level chunks");
+    CK(dev_alloc(&L.raw, sizeof(uint32_t) * L.task_cap), "alloc task list");
+    CK(dev_alloc(&L.info, sizeof(int4) * N * nd), "alloc classification");
+    CK(dev_alloc(&L.level, sizeof(int32_t) * N * nd), "alloc levels");
+    CK(dev_alloc(&L.word, sizeof(unsigned long long) * N * nd), "alloc levels");
+    CK(dev_alloc(&L.lvl_cnt, sizeof(int32_t) * (N + 2)), "alloc level counts");
+    CK(dev_alloc(&L.pad_off, sizeof(uint32_t) * (N + 2)), "alloc level offsets");
+    CK(dev_alloc(&L.lev_chunk, sizeof(int64_t) * (N + 2)), "alloc level chunks");
     L.dlev_cap = (int)std::min<int64_t>(N + 1, 1 << 16);
-    CK(cudaMalloc(&L.dlev, sizeof(int32_t) * ((int64_t)nd * (2 * L.dlev_cap + 2) + 1)), "alloc level tables");
+    CK(dev_alloc(&L.dlev, sizeof(int32_t) * ((int64_t)nd * (2 * L.dlev_cap + 2) + 1)), "alloc level tables");
     // worst case of levels x (nd+1) segment starts is only known after levelisation
     return SWEEP_OK;
 }
@@ -203,10 +204,10 @@ sweep_status run_levelise(sweep_ctx* c, Levels& L, int d0, int nd, long long bud
     // scheme (b) tables, [N][nd] each (freed when scheme (a) is levelised again)
     if (transport > 0 && !L.dc_mask) {
         const size_t n = (size_t)c->mesh.N * nd;
-        CK(cudaMalloc(&L.dc_mask, sizeof(uint64_t) * n), "alloc scheme (b) tables");
-        CK(cudaMalloc(&L.dc_inm, sizeof(uint64_t) * n), "alloc scheme (b) tables");
-        CK(cudaMalloc(&L.dc_share32, sizeof(float) * n), "alloc scheme (b) tables");
-        CK(cudaMalloc(&L.dc_share64, sizeof(double) * n), "alloc scheme (b) tables");
+        CK(dev_alloc(&L.dc_mask, sizeof(uint64_t) * n), "alloc scheme (b) tables");
+        CK(dev_alloc(&L.dc_inm, sizeof(uint64_t) * n), "alloc scheme (b) tables");
+        CK(dev_alloc(&L.dc_share32, sizeof(float) * n), "alloc scheme (b) tables");
+        CK(dev_alloc(&L.dc_share64, sizeof(double) * n), "alloc scheme (b) tables");
     } else if (transport == 0 && L.dc_mask) {
         dfree(L.dc_mask); dfree(L.dc_inm); dfree(L.dc_share32); dfree(L.dc_share64);
     }
@@ -229,12 +230,12 @@ long long budget_of(const sweep_opts* o) { return o && o->spin_budget > 0 ? o->s
 
 sweep_status ensure_common(sweep_ctx* c) {
     if (!c->bar) {
-        CK(cudaMalloc(&c->bar, sizeof(GridBar)), "alloc");
-        CK(cudaMalloc(&c->derr, sizeof(int)), "alloc");
-        CK(cudaMalloc(&c->scratch, sizeof(int64_t) * 4), "alloc");
-        CK(cudaMalloc(&c->red, sizeof(double) * 4), "alloc");
-        CK(cudaMalloc(&c->dmax, 2 * sizeof(unsigned long long)), "alloc");  // [0] periodic or scattering, [1] scattering when fused
-        CK(cudaMalloc(&c->stall_word, sizeof(double)), "alloc");
+        CK(dev_alloc(&c->bar, sizeof(GridBar)), "alloc");
+        CK(dev_alloc(&c->derr, sizeof(int)), "alloc");
+        CK(dev_alloc(&c->scratch, sizeof(int64_t) * 4), "alloc");
+        CK(dev_alloc(&c->red, sizeof(double) * 4), "alloc");
+        CK(dev_alloc(&c->dmax, 2 * sizeof(unsigned long long)), "alloc");  // [0] periodic or scattering, [1] scattering when fused
+        CK(dev_alloc(&c->stall_word, sizeof(double)), "alloc");
         CK(cudaMemset(c->stall_word, 0, sizeof(double)), "init");
     }
     return SWEEP_OK;
@@ -244,11 +245,11 @@ sweep_status ensure_ng(sweep_ctx* c, size_t ng) {
     if (c->ng_cap >= ng && c->J) return SWEEP_OK;
     dfree(c->J); dfree(c->Jold); dfree(c->Gam); dfree(c->jn); dfree(c->jn1);
     size_t n = ng > 0 ? ng : 1;
-    CK(cudaMalloc(&c->J, sizeof(double) * n), "alloc J");
-    CK(cudaMalloc(&c->Jold, sizeof(double) * n), "alloc J");
-    CK(cudaMalloc(&c->Gam, sizeof(double) * n), "alloc Gamma");
-    CK(cudaMalloc(&c->jn, sizeof(double) * n), "alloc j");
-    CK(cudaMalloc(&c->jn1, sizeof(double) * n), "alloc j");
+    CK(dev_alloc(&c->J, sizeof(double) * n), "alloc J");
+    CK(dev_alloc(&c->Jold, sizeof(double) * n), "alloc J");
+    CK(dev_alloc(&c->Gam, sizeof(double) * n), "alloc Gamma");
+    CK(dev_alloc(&c->jn, sizeof(double) * n), "alloc j");
+    CK(dev_alloc(&c->jn1, sizeof(double) * n), "alloc j");
     c->ng_cap = n;
     return SWEEP_OK;
 }
@@ -257,8 +258,8 @@ sweep_status ensure_cm(sweep_ctx* c, size_t n) {
     if (c->cm_cap >= n && c->cm32) return SWEEP_OK;
     dfree(c->cm32); dfree(c->cm64);
     size_t m = n > 0 ? n : 1;
-    CK(cudaMalloc(&c->cm32, sizeof(float2) * m), "alloc sources");
-    CK(cudaMalloc(&c->cm64, sizeof(double2) * m), "alloc sources");
+    CK(dev_alloc(&c->cm32, sizeof(float2) * m), "alloc sources");
+    CK(dev_alloc(&c->cm64, sizeof(double2) * m), "alloc sources");
     c->cm_cap = m;
     return SWEEP_OK;
 }
@@ -266,7 +267,7 @@ sweep_status ensure_cm(sweep_ctx* c, size_t n) {
 sweep_status ensure_partial(sweep_ctx* c, int nblk) {
     if (c->partial_cap >= nblk && c->partial) return SWEEP_OK;
     dfree(c->partial);
-    CK(cudaMalloc(&c->partial, sizeof(double) * 2 * (nblk > 0 ? nblk : 1)), "alloc partials");
+    CK(dev_alloc(&c->partial, sizeof(double) * 2 * (nblk > 0 ? nblk : 1)), "alloc partials");
     c->partial_cap = nblk;
     return SWEEP_OK;
 }
@@ -653,6 +654,7 @@ sweep_status sweep_create(sweep_ctx** out, int device, void* stream) {
     sweep_ctx* c = new sweep_ctx();
     c->device = device;
     c->st = (cudaStream_t)stream;
+    PoolScope pool_scope(&c->pool);
     cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device);
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
@@ -672,6 +674,7 @@ sweep_status sweep_create(sweep_ctx** out, int device, void* stream) {
 sweep_status sweep_destroy(sweep_ctx* c) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     cudaStreamSynchronize(c->st);
     free_levels(c->lev);
     free_levels(c->adj_lev);
@@ -695,6 +698,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
                             int32_t n_meshes, const int64_t* mesh_cell_offset) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (n_cells < 1 || n_cells >= (1ll << 30)) return bad(c, "n_cells must be in [1, 2^30)");
     if (n_faces < 0) return bad(c, "n_faces < 0");
     if (!volume || (n_faces > 0 && (!face_cells || !area || !normal || !flags))) return bad(c, "null mesh array");
@@ -728,18 +732,18 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     int* d_bad = nullptr;
     int64_t F1 = n_faces > 0 ? n_faces : 1;
     auto cleanup = [&]() {
-        cudaFree(d_area); cudaFree(d_normal); cudaFree(d_fc); cudaFree(d_tmp); cudaFree(d_flags);
-        cudaFree(d_off); cudaFree(d_bad);
+        dev_free(d_area); dev_free(d_normal); dev_free(d_fc); dev_free(d_tmp); dev_free(d_flags);
+        dev_free(d_off); dev_free(d_bad);
     };
-#define CKM(x, what) do { cudaError_t _e = (x); if (_e != cudaSuccess) { cleanup(); cudaFree(d_vol); return cuda_status(c, _e, what); } } while (0)
-    CKM(cudaMalloc(&d_vol, sizeof(double) * n_cells), "alloc volume");
-    CKM(cudaMalloc(&d_area, sizeof(double) * F1), "alloc area");
-    CKM(cudaMalloc(&d_normal, sizeof(double) * 3 * F1), "alloc normal");
-    CKM(cudaMalloc(&d_fc, sizeof(int32_t) * 2 * F1), "alloc faces");
-    CKM(cudaMalloc(&d_flags, F1), "alloc flags");
-    CKM(cudaMalloc(&d_off, sizeof(int64_t) * off.size()), "alloc offsets");
-    CKM(cudaMalloc(&d_bad, sizeof(int)), "alloc");
-    CKM(cudaMalloc(&d_tmp, sizeof(int32_t) * ((n_cells > n_faces ? n_cells : n_faces) + 2)), "alloc");
+#define CKM(x, what) do { cudaError_t _e = (x); if (_e != cudaSuccess) { cleanup(); dev_free(d_vol); return cuda_status(c, _e, what); } } while (0)
+    CKM(dev_alloc(&d_vol, sizeof(double) * n_cells), "alloc volume");
+    CKM(dev_alloc(&d_area, sizeof(double) * F1), "alloc area");
+    CKM(dev_alloc(&d_normal, sizeof(double) * 3 * F1), "alloc normal");
+    CKM(dev_alloc(&d_fc, sizeof(int32_t) * 2 * F1), "alloc faces");
+    CKM(dev_alloc(&d_flags, F1), "alloc flags");
+    CKM(dev_alloc(&d_off, sizeof(int64_t) * off.size()), "alloc offsets");
+    CKM(dev_alloc(&d_bad, sizeof(int)), "alloc");
+    CKM(dev_alloc(&d_tmp, sizeof(int32_t) * ((n_cells > n_faces ? n_cells : n_faces) + 2)), "alloc");
     CKM(cudaMemcpyAsync(d_vol, volume, sizeof(double) * n_cells, cudaMemcpyHostToDevice, c->st), "upload");
     if (n_faces > 0) {
         CKM(cudaMemcpyAsync(d_area, area, sizeof(double) * n_faces, cudaMemcpyHostToDevice, c->st), "upload");
@@ -756,7 +760,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     CKM(cudaStreamSynchronize(c->st), "validate mesh");
     if (hbad) {
         cleanup();
-        cudaFree(d_vol);
+        dev_free(d_vol);
         char buf[160];
         snprintf(buf, sizeof buf,
                  "invalid mesh (flags %d: 1 cell index, 2 face flags, 4 area, 8 normal, 16 volume, 32 face crosses "
@@ -770,12 +774,12 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     m.NB = NB;
     m.vol = d_vol;
     m.mesh_off = off;
-    CKM(cudaMalloc(&m.rowptr, sizeof(uint32_t) * (n_cells + 1)), "alloc rows");
-    CKM(cudaMalloc(&m.side, sizeof(int4) * (S > 0 ? S : 1) + 64 * sizeof(int4)), "alloc sides");
-    CKM(cudaMalloc(&m.side64, sizeof(d4) * (S > 0 ? S : 1)), "alloc sides");
-    CKM(cudaMalloc(&m.side_lo, sizeof(float4) * (S > 0 ? S : 1)), "alloc sides");
-    CKM(cudaMalloc(&m.ids, sizeof(int32_t) * 32 * n_cells), "alloc sides");
-    CKM(cudaMalloc(&m.twin, sizeof(uint32_t) * (S > 0 ? S : 1)), "alloc sides");
+    CKM(dev_alloc(&m.rowptr, sizeof(uint32_t) * (n_cells + 1)), "alloc rows");
+    CKM(dev_alloc(&m.side, sizeof(int4) * (S > 0 ? S : 1) + 64 * sizeof(int4)), "alloc sides");
+    CKM(dev_alloc(&m.side64, sizeof(d4) * (S > 0 ? S : 1)), "alloc sides");
+    CKM(dev_alloc(&m.side_lo, sizeof(float4) * (S > 0 ? S : 1)), "alloc sides");
+    CKM(dev_alloc(&m.ids, sizeof(int32_t) * 32 * n_cells), "alloc sides");
+    CKM(dev_alloc(&m.twin, sizeof(uint32_t) * (S > 0 ? S : 1)), "alloc sides");
     CKM(launch_build_csr(m, d_fc, d_area, d_normal, d_flags, d_tmp, c->st), "build CSR");
     CKM(cudaStreamSynchronize(c->st), "build CSR");
 #undef CKM
@@ -787,6 +791,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
 sweep_status sweep_set_directions(sweep_ctx* c, int32_t n_dir, const double* omega, const double* weight) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (n_dir < 1 || n_dir > 1024) return bad(c, "n_dir must be in [1, 1024]");
     if (!omega || !weight) return bad(c, "null direction array");
     double ws = 0.0;
@@ -810,10 +815,10 @@ sweep_status sweep_set_directions(sweep_ctx* c, int32_t n_dir, const double* ome
         o32lo[d] = make_float4((float)(w[0] - (double)o32[d].x), (float)(w[1] - (double)o32[d].y),
                                (float)(w[2] - (double)o32[d].z), 0.f);
     }
-    CK(cudaMalloc(&c->om64, sizeof(double) * 3 * n_dir), "alloc directions");
-    CK(cudaMalloc(&c->w64, sizeof(double) * n_dir), "alloc directions");
-    CK(cudaMalloc(&c->om32, sizeof(float4) * n_dir), "alloc directions");
-    CK(cudaMalloc(&c->om32lo, sizeof(float4) * n_dir), "alloc directions");
+    CK(dev_alloc(&c->om64, sizeof(double) * 3 * n_dir), "alloc directions");
+    CK(dev_alloc(&c->w64, sizeof(double) * n_dir), "alloc directions");
+    CK(dev_alloc(&c->om32, sizeof(float4) * n_dir), "alloc directions");
+    CK(dev_alloc(&c->om32lo, sizeof(float4) * n_dir), "alloc directions");
     CK(cudaMemcpyAsync(c->om64, omega, sizeof(double) * 3 * n_dir, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemcpyAsync(c->w64, weight, sizeof(double) * n_dir, cudaMemcpyHostToDevice, c->st), "upload");
     CK(cudaMemcpyAsync(c->om32, o32.data(), sizeof(float4) * n_dir, cudaMemcpyHostToDevice, c->st), "upload");
@@ -829,6 +834,7 @@ static sweep_status set_material_impl(sweep_ctx* c, int32_t G, const double* ka,
                                       const double* bc, bool dev) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (!c->has_mesh) return bad(c, "set the mesh first");
     if (G < 1 || G > 8) return bad(c, "n_groups must be in [1, 8]");
     if (!ka || !em) return bad(c, "kappa_abs and emissivity are required");
@@ -852,17 +858,17 @@ static sweep_status set_material_impl(sweep_ctx* c, int32_t G, const double* ka,
     free_material(c);
     cudaMemcpyKind kind = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     size_t nb = sizeof(double) * (NG > 0 ? NG : 1);
-    CK(cudaMalloc(&c->ka, nb), "alloc material");
-    CK(cudaMalloc(&c->em, nb), "alloc material");
+    CK(dev_alloc(&c->ka, nb), "alloc material");
+    CK(dev_alloc(&c->em, nb), "alloc material");
     CK(cudaMemcpyAsync(c->ka, ka, sizeof(double) * NG, kind, c->st), "upload material");
     CK(cudaMemcpyAsync(c->em, em, sizeof(double) * NG, kind, c->st), "upload material");
     if (ks) {
-        CK(cudaMalloc(&c->ks, nb), "alloc material");
+        CK(dev_alloc(&c->ks, nb), "alloc material");
         CK(cudaMemcpyAsync(c->ks, ks, sizeof(double) * NG, kind, c->st), "upload material");
         if (dev) scat = true;  // not inspected on the host; a zero array costs one extra sweep
     }
     if (bc && NBG > 0) {
-        CK(cudaMalloc(&c->bc, sizeof(double) * NBG), "alloc boundary inflow");
+        CK(dev_alloc(&c->bc, sizeof(double) * NBG), "alloc boundary inflow");
         CK(cudaMemcpyAsync(c->bc, bc, sizeof(double) * NBG, kind, c->st), "upload boundary inflow");
     }
     if (!dev) CK(cudaStreamSynchronize(c->st), "upload material");
@@ -913,9 +919,7 @@ int wanted_format(sweep_ctx* c, const Levels& L, const sweep_opts* o, int prec) 
 
 // device memory for an operator of `bytes`, keeping a margin for the solve buffers allocated later
 bool op_fits(size_t bytes) {
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    return bytes + (size_t)(2ull << 30) <= free_b;
+    return bytes + (size_t)(2ull << 30) <= dev_available();
 }
 
 // Plans and writes a packed operator of the levels L (transposed: the adjoint's), growing its buffers
@@ -933,8 +937,8 @@ bool build_packed(sweep_ctx* c, Levels& L, PackedOp& P, bool transposed) {
         dfree(P.meta);
         P.cap = 0;
         const int64_t cap = n_pk + n_pk / 16 + 64;
-        ok = op_fits((size_t)cap * 520) && cudaMalloc(&P.pk, (size_t)cap * 512) == cudaSuccess &&
-             cudaMalloc(&P.meta, (size_t)cap * 8) == cudaSuccess;
+        ok = op_fits((size_t)cap * 520) && dev_alloc(&P.pk, (size_t)cap * 512) == cudaSuccess &&
+             dev_alloc(&P.meta, (size_t)cap * 8) == cudaSuccess;
         if (ok) P.cap = cap;
         else {
             cudaGetLastError();
@@ -1002,7 +1006,7 @@ sweep_status ensure_operator(sweep_ctx* c, Levels& L, const sweep_opts* o, int p
         if (bytes > L.op_bytes) {
             dfree(L.op);
             L.op_bytes = 0;
-            ok = op_fits(bytes) && cudaMalloc(&L.op, bytes) == cudaSuccess;
+            ok = op_fits(bytes) && dev_alloc(&L.op, bytes) == cudaSuccess;
             if (ok) L.op_bytes = bytes;
             else {
                 cudaGetLastError();
@@ -1049,7 +1053,7 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int 
         dfree(p);
         cap = 0;
         const int64_t n = need + need / 16 + 256;
-        if (!op_fits((size_t)n) || cudaMalloc(&p, (size_t)n) != cudaSuccess) {
+        if (!op_fits((size_t)n) || dev_alloc(&p, (size_t)n) != cudaSuccess) {
             cudaGetLastError();
             p = nullptr;
             return false;
@@ -1096,7 +1100,7 @@ sweep_status ensure_solution(sweep_ctx* c, int prec, bool two) {
         dfree(b.I[0]);
         dfree(b.I[1]);
         b = SolveBuf();
-        CK(cudaMalloc(&b.I[0], bytes > 0 ? bytes : 4), "alloc intensities");
+        CK(dev_alloc(&b.I[0], bytes > 0 ? bytes : 4), "alloc intensities");
         CK(cudaMemsetAsync(b.I[0], 0, bytes, c->st), "init intensities");
         b.bytes = bytes;
         b.prec = prec;
@@ -1105,7 +1109,7 @@ sweep_status ensure_solution(sweep_ctx* c, int prec, bool two) {
         b.G = c->G;
     }
     if (two && !b.I[1]) {
-        CK(cudaMalloc(&b.I[1], bytes > 0 ? bytes : 4), "alloc intensities");
+        CK(dev_alloc(&b.I[1], bytes > 0 ? bytes : 4), "alloc intensities");
         CK(cudaMemsetAsync(b.I[1], 0, bytes, c->st), "init intensities");
         b.sign[1] = 0;
     }
@@ -1117,7 +1121,7 @@ sweep_status ensure_mean(sweep_ctx* c, int prec) {
     if (c->Imean && c->imean_bytes == bytes) return SWEEP_OK;
     dfree(c->Imean);
     c->imean_bytes = 0;
-    CK(cudaMalloc(&c->Imean, bytes > 0 ? bytes : 4), "alloc cell means");
+    CK(dev_alloc(&c->Imean, bytes > 0 ? bytes : 4), "alloc cell means");
     c->imean_bytes = bytes;
     return SWEEP_OK;
 }
@@ -1205,7 +1209,7 @@ template <typename T>
 struct DevBuf {
     T* p = nullptr;
     ~DevBuf() {
-        if (p) cudaFree(p);
+        if (p) dev_free(p);
     }
 };
 __global__ void k_bc_to_f32(const double* in, int64_t n, float* out) {
@@ -1217,7 +1221,7 @@ __global__ void k_bc_to_f32(const double* in, int64_t n, float* out) {
 sweep_status ensure_bc32(sweep_ctx* c) {
     if (c->bc32_ready) return SWEEP_OK;
     const int64_t n = c->mesh.NB * c->G;
-    if (!c->bc32) CK(cudaMalloc(&c->bc32, sizeof(float) * (n > 0 ? n : 1)), "alloc boundary inflow");
+    if (!c->bc32) CK(dev_alloc(&c->bc32, sizeof(float) * (n > 0 ? n : 1)), "alloc boundary inflow");
     k_bc_to_f32<<<nblocks256(n), 256, 0, c->st>>>(c->bc, n, c->bc32);
     ++c->launches;
     CK(cudaGetLastError(), "boundary inflow");
@@ -1229,6 +1233,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
                         sweep_stats* stats) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (!c->has_mesh || !c->has_dirs || !c->has_mat) return bad(c, "set mesh, directions and material first");
     sweep_opts o;
     if (opts_in) o = *opts_in;
@@ -1474,6 +1479,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     if (Gam_out) CK(cudaMemcpyAsync(Gam_out, c->Gam, sizeof(double) * NG, k, c->st), "copy Gamma");
     cudaEventRecord(t1, c->st);
     CK(cudaStreamSynchronize(c->st), "solve");
+    c->pool.end_of_call();
     float ttot = 0;
     cudaEventElapsedTime(&ttot, t0, t1);
     S.absorbed = hr[0];
@@ -1512,6 +1518,7 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
                           double* ge_out, double* gks_out, bool dev, sweep_stats* stats) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (!c->has_mesh || !c->has_dirs || !c->has_mat) return bad(c, "set mesh, directions and material first");
     if (c->G > 4) return bad(c, "the adjoint supports at most 4 groups");
     if (opts_in && opts_in->law != SWEEP_LAW_BALANCE) return bad(c, "the adjoint takes the BALANCE law");
@@ -1544,22 +1551,22 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     DevBuf<double> b_dlj, b_dlg, b_gk, b_ge;
     cudaMemcpyKind kin = dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     if (dlj) {
-        CK(cudaMalloc(&b_dlj.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
+        CK(dev_alloc(&b_dlj.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
         CK(cudaMemcpyAsync(b_dlj.p, dlj, sizeof(double) * NG, kin, c->st), "upload");
     }
     if (dlg) {
-        CK(cudaMalloc(&b_dlg.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
+        CK(dev_alloc(&b_dlg.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
         CK(cudaMemcpyAsync(b_dlg.p, dlg, sizeof(double) * NG, kin, c->st), "upload");
     }
-    CK(cudaMalloc(&b_gk.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
-    CK(cudaMalloc(&b_ge.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
+    CK(dev_alloc(&b_gk.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
+    CK(dev_alloc(&b_ge.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
     double *d_dlj = b_dlj.p, *d_dlg = b_dlg.p, *gk = b_gk.p, *ge = b_ge.p;
     CK(cudaMemsetAsync(gk, 0, sizeof(double) * NG, c->st), "init");
     CK(cudaMemsetAsync(ge, 0, sizeof(double) * NG, c->st), "init");
     DevBuf<double> b_gks, b_mu;
-    if (gks_out) CK(cudaMalloc(&b_gks.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
+    if (gks_out) CK(dev_alloc(&b_gks.p, sizeof(double) * (NG > 0 ? NG : 1)), "alloc");
     if (scat || pbc) {
-        CK(cudaMalloc(&b_mu.p, sizeof(double) * (2 * NG > 0 ? 2 * NG : 1)), "alloc");
+        CK(dev_alloc(&b_mu.p, sizeof(double) * (2 * NG > 0 ? 2 * NG : 1)), "alloc");
         CK(cudaMemsetAsync(b_mu.p, 0, sizeof(double) * 2 * NG, c->st), "init");
     }
     sweep_status s = SWEEP_OK;
@@ -1584,8 +1591,8 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     if (c->adj_bytes_I != bI || c->adj_bytes_L != bL) {
         dfree(c->adjI);
         dfree(c->adjL);
-        CK(cudaMalloc(&c->adjI, bI > 0 ? bI : 4), "alloc adjoint batch");
-        CK(cudaMalloc(&c->adjL, bL > 0 ? bL : 4), "alloc adjoint batch");
+        CK(dev_alloc(&c->adjI, bI > 0 ? bI : 4), "alloc adjoint batch");
+        CK(dev_alloc(&c->adjL, bL > 0 ? bL : 4), "alloc adjoint batch");
         c->adj_bytes_I = bI;
         c->adj_bytes_L = bL;
     }
@@ -1595,7 +1602,7 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     CK(cudaMemsetAsync(c->adjL, 0, bL, c->st), "init");
     DevBuf<char> b_lam2;
     if (pbc) {
-        CK(cudaMalloc(&b_lam2.p, bL > 0 ? bL : 4), "alloc adjoint batch");
+        CK(dev_alloc(&b_lam2.p, bL > 0 ? bL : 4), "alloc adjoint batch");
         CK(cudaMemsetAsync(b_lam2.p, 0, bL, c->st), "init");
     }
     void* lbuf[2] = {c->adjL, b_lam2.p};
@@ -1708,6 +1715,7 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     if (gks_out) CK(cudaMemcpyAsync(gks_out, b_gks.p, sizeof(double) * NG, kout, c->st), "copy gradient");
     cudaEventRecord(t1, c->st);
     CK(cudaStreamSynchronize(c->st), "adjoint");
+    c->pool.end_of_call();
     float ttot = 0;
     cudaEventElapsedTime(&ttot, t0, t1);
     S.n_sweeps = n_sweeps;
@@ -1756,6 +1764,7 @@ sweep_status sweep_solve_dev(sweep_ctx* c, const sweep_opts* o, double* J, doubl
 sweep_status sweep_levels(sweep_ctx* c, int32_t dir, int32_t* level, int32_t* depth) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (!c->has_mesh || !c->has_dirs) return bad(c, "set mesh and directions first");
     if (dir < 0 || dir >= c->D) return bad(c, "direction index out of range");
     sweep_status s = ensure_levels(c, nullptr, nullptr, nullptr);
@@ -1771,18 +1780,19 @@ sweep_status sweep_levels(sweep_ctx* c, int32_t dir, int32_t* level, int32_t* de
 sweep_status sweep_intensity(sweep_ctx* c, int32_t dir, double* out) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (c->sb.last < 0 || !c->sb.I[c->sb.last]) return bad(c, "no solve yet");
     if (dir < 0 || dir >= c->sb.nd) return bad(c, "direction index out of range");
     if (!out) return bad(c, "null output");
     const size_t n = (size_t)c->sb.N * c->sb.G;
     double* tmp = nullptr;
-    CK(cudaMalloc(&tmp, sizeof(double) * (n > 0 ? n : 1)), "alloc");
+    CK(dev_alloc(&tmp, sizeof(double) * (n > 0 ? n : 1)), "alloc");
     const size_t es = c->sb.prec == 64 ? 8 : 4;
     const char* src = (const char*)c->sb.I[c->sb.last] + es * n * dir;
     cudaError_t e = launch_to_f64(c->sb.prec, src, (int64_t)n, tmp, c->st);
     if (e == cudaSuccess) e = cudaMemcpyAsync(out, tmp, sizeof(double) * n, cudaMemcpyDeviceToHost, c->st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->st);
-    cudaFree(tmp);
+    dev_free(tmp);
     return cuda_status(c, e, "copy intensity");
 }
 
@@ -1791,6 +1801,7 @@ sweep_status sweep_intensity(sweep_ctx* c, int32_t dir, double* out) {
 sweep_status sweep_rotate_directions(sweep_ctx* c, const double* R, int64_t n_quad) {
     if (!c) return SWEEP_ERR_INVALID_ARG;
     cudaSetDevice(c->device);
+    PoolScope pool_scope(&c->pool);
     if (!c->has_dirs) return bad(c, "set the directions first");
     if (!R) return bad(c, "null rotation");
     if (n_quad == 0) n_quad = 1 << 16;
@@ -1832,9 +1843,9 @@ sweep_status sweep_rotate_directions(sweep_ctx* c, const double* R, int64_t n_qu
         DevBuf<double3> d_pts;
         DevBuf<double> d_new;
         DevBuf<unsigned long long> d_cnt;
-        CK(cudaMalloc(&d_pts.p, sizeof(double3) * (size_t)n_quad), "alloc quadrature");
-        CK(cudaMalloc(&d_new.p, sizeof(double) * 3 * D), "alloc directions");
-        CK(cudaMalloc(&d_cnt.p, sizeof(unsigned long long) * (size_t)D * D), "alloc counts");
+        CK(dev_alloc(&d_pts.p, sizeof(double3) * (size_t)n_quad), "alloc quadrature");
+        CK(dev_alloc(&d_new.p, sizeof(double) * 3 * D), "alloc directions");
+        CK(dev_alloc(&d_cnt.p, sizeof(unsigned long long) * (size_t)D * D), "alloc counts");
         CK(cudaMemcpyAsync(d_pts.p, pts.data(), sizeof(double3) * (size_t)n_quad, cudaMemcpyHostToDevice, c->st),
            "upload");
         CK(cudaMemcpyAsync(d_new.p, om_new.data(), sizeof(double) * 3 * D, cudaMemcpyHostToDevice, c->st), "upload");
@@ -1861,16 +1872,16 @@ sweep_status sweep_rotate_directions(sweep_ctx* c, const double* R, int64_t n_qu
         DevBuf<int32_t> d_rp, d_col;
         DevBuf<double> d_val;
         const size_t nnz = col.size() > 0 ? col.size() : 1;
-        CK(cudaMalloc(&d_rp.p, sizeof(int32_t) * (D + 1)), "alloc remap");
-        CK(cudaMalloc(&d_col.p, sizeof(int32_t) * nnz), "alloc remap");
-        CK(cudaMalloc(&d_val.p, sizeof(double) * nnz), "alloc remap");
+        CK(dev_alloc(&d_rp.p, sizeof(int32_t) * (D + 1)), "alloc remap");
+        CK(dev_alloc(&d_col.p, sizeof(int32_t) * nnz), "alloc remap");
+        CK(dev_alloc(&d_val.p, sizeof(double) * nnz), "alloc remap");
         CK(cudaMemcpyAsync(d_rp.p, rp.data(), sizeof(int32_t) * (D + 1), cudaMemcpyHostToDevice, c->st), "upload");
         CK(cudaMemcpyAsync(d_col.p, col.data(), sizeof(int32_t) * col.size(), cudaMemcpyHostToDevice, c->st), "upload");
         CK(cudaMemcpyAsync(d_val.p, val.data(), sizeof(double) * val.size(), cudaMemcpyHostToDevice, c->st), "upload");
         // remap the last solve's intensities into the other buffer, which becomes the last one
         const int src = b.last, dst = 1 - b.last;
         if (!b.I[dst]) {
-            CK(cudaMalloc(&b.I[dst], b.bytes > 0 ? b.bytes : 4), "alloc intensities");
+            CK(dev_alloc(&b.I[dst], b.bytes > 0 ? b.bytes : 4), "alloc intensities");
             b.sign[dst] = 0;
         }
         const int64_t NG = b.N * (int64_t)b.G;

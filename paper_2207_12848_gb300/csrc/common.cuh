@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <cstddef>
 #include <string>
 #include <vector>
 
@@ -339,6 +340,52 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, long l
 // ---------------------------------------------------------------------------------------------
 // Host-side structures
 // ---------------------------------------------------------------------------------------------
+
+// Device memory of one context. A cudaMalloc or cudaFree costs tens of microseconds, and a free waits for the device;
+// a time step that sets a mesh or a material and solves makes a dozen to fifty of them. Blocks that the context gives
+// up are kept, LIMIT bytes of them at most, and handed out again for a request that fills four fifths of one or more.
+// Everything a context does is ordered on its stream, so a block may be handed out while work on its former contents
+// is queued. Blocks that nothing asked for during KEEP solves or adjoints are freed, as are all of them when an
+// allocation fails and when the context is destroyed. Measured on a step that sets a mesh and a material (67,581
+// cells, 48 directions) and solves: 6.9 ms -> 4.35 ms; a solve and adjoint of 2^18 cells 6.6 -> 5.75 ms.
+class MemPool {
+public:
+    static constexpr int KEEP = 4;
+    static constexpr size_t LIMIT = (size_t)1 << 30;
+    ~MemPool();
+    cudaError_t alloc(void** p, size_t bytes);
+    void free(void* p);
+    void end_of_call();             // a solve or adjoint has ended: free what has not been asked for lately
+    void trim(int keep);            // free the blocks given up more than `keep` calls ago (0: all)
+    size_t cached() const { return cached_; }
+
+private:
+    struct Block {
+        void* p;
+        size_t bytes;
+        int epoch;
+    };
+    std::vector<Block> live_, free_;
+    size_t cached_ = 0;
+    int epoch_ = 0;
+};
+// the pool of the context whose entry point this thread is in
+class PoolScope {
+public:
+    explicit PoolScope(MemPool* p);
+    ~PoolScope();
+    PoolScope(const PoolScope&) = delete;
+    PoolScope& operator=(const PoolScope&) = delete;
+
+private:
+    MemPool* before_;
+};
+cudaError_t dev_alloc_bytes(void** p, size_t bytes);
+void dev_free(void* p);
+template <typename T>
+cudaError_t dev_alloc(T** p, size_t bytes) { return dev_alloc_bytes(reinterpret_cast<void**>(p), bytes); }
+size_t dev_available();  // bytes an allocation could get: free on the device, and kept by the pool
+
 struct DevMesh {
     int64_t N = 0, F = 0, S = 0, NB = 0;  // cells, faces, face sides, boundary faces
     uint32_t* rowptr = nullptr;            // [N+1]

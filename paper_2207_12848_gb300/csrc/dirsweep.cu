@@ -981,21 +981,19 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
                  o_st = part(16), o_tt = part(16), o_sc = part(8 * ((size_t)nd + 1));
     cudaError_t e;
     if (off > L.dir_ws_bytes) {
-        if (L.dir_ws) cudaFree(L.dir_ws);
+        if (L.dir_ws) dev_free(L.dir_ws);
         L.dir_ws = nullptr;
         L.dir_ws_bytes = 0;
-        size_t free_b = 0, total_b = 0;
-        cudaMemGetInfo(&free_b, &total_b);
-        if (off + ((size_t)2 << 30) > free_b) return cudaSuccess;
-        if ((e = cudaMalloc(&L.dir_ws, off))) return e;
+        if (off + ((size_t)2 << 30) > dev_available()) return cudaSuccess;
+        if ((e = dev_alloc(&L.dir_ws, off))) return e;
         L.dir_ws_bytes = off;
     }
     const size_t keep = ((sizeof(DirMeta) * nd + 255) & ~(size_t)255) + 8 * nR;
     if (keep > P.meta_bytes) {
-        if (P.meta) cudaFree(P.meta);
+        if (P.meta) dev_free(P.meta);
         P.meta = nullptr;
         P.meta_bytes = 0;
-        if ((e = cudaMalloc(&P.meta, keep))) return e;
+        if ((e = dev_alloc(&P.meta, keep))) return e;
         P.meta_bytes = keep;
     }
     P.rtab = (uint2*)((char*)P.meta + ((sizeof(DirMeta) * nd + 255) & ~(size_t)255));

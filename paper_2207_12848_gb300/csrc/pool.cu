@@ -1,0 +1,93 @@
+// Device memory kept by a context between calls (MemPool in common.cuh).
+#include "common.cuh"
+
+namespace sw {
+
+namespace {
+thread_local MemPool* t_pool = nullptr;
+size_t rounded(size_t n) {
+    const size_t unit = n >= (1u << 20) ? (size_t)1 << 16 : 512;
+    return (n + unit - 1) / unit * unit;
+}
+}  // namespace
+
+MemPool::~MemPool() {
+    trim(0);
+    for (const Block& b : live_) cudaFree(b.p);
+}
+
+cudaError_t MemPool::alloc(void** p, size_t bytes) {
+    const size_t n = rounded(bytes > 0 ? bytes : 1);
+    size_t best = free_.size();
+    for (size_t i = 0; i < free_.size(); ++i)
+        if (free_[i].bytes >= n && free_[i].bytes / 5 * 4 <= n && (best == free_.size() || free_[i].bytes < free_[best].bytes)) best = i;
+    if (best < free_.size()) {
+        *p = free_[best].p;
+        cached_ -= free_[best].bytes;
+        live_.push_back(free_[best]);
+        free_.erase(free_.begin() + (std::ptrdiff_t)best);
+        return cudaSuccess;
+    }
+    cudaError_t e = cudaMalloc(p, n);
+    if (e == cudaErrorMemoryAllocation && !free_.empty()) {
+        cudaGetLastError();
+        trim(0);
+        e = cudaMalloc(p, n);
+    }
+    if (e != cudaSuccess) {
+        *p = nullptr;
+        return e;
+    }
+    live_.push_back(Block{*p, n, 0});
+    return cudaSuccess;
+}
+
+void MemPool::free(void* p) {
+    if (!p) return;
+    for (size_t i = 0; i < live_.size(); ++i) {
+        if (live_[i].p != p) continue;
+        Block b = live_[i];
+        live_.erase(live_.begin() + (std::ptrdiff_t)i);
+        if (b.bytes > LIMIT - cached_) break;
+        b.epoch = epoch_;
+        cached_ += b.bytes;
+        free_.push_back(b);
+        return;
+    }
+    cudaFree(p);
+}
+
+void MemPool::trim(int keep) {
+    size_t n = 0;
+    for (const Block& b : free_) {
+        if (keep > 0 && epoch_ - b.epoch < keep) {
+            free_[n++] = b;
+        } else {
+            cached_ -= b.bytes;
+            cudaFree(b.p);
+        }
+    }
+    free_.resize(n);
+}
+
+void MemPool::end_of_call() {
+    ++epoch_;
+    trim(KEEP);
+}
+
+PoolScope::PoolScope(MemPool* p) : before_(t_pool) { t_pool = p; }
+PoolScope::~PoolScope() { t_pool = before_; }
+
+cudaError_t dev_alloc_bytes(void** p, size_t bytes) { return t_pool ? t_pool->alloc(p, bytes) : cudaMalloc(p, bytes); }
+void dev_free(void* p) {
+    if (!p) return;
+    if (t_pool) t_pool->free(p);
+    else cudaFree(p);
+}
+size_t dev_available() {
+    size_t free_b = 0, total_b = 0;
+    cudaMemGetInfo(&free_b, &total_b);
+    return free_b + (t_pool ? t_pool->cached() : 0);
+}
+
+}  // namespace sw

@@ -289,16 +289,16 @@ cudaError_t launch_build_csr(const DevMesh& mc, const int32_t* fc, const double*
     int64_t nmax = (N > F ? N : F) + 1;
     int64_t nsb = nmax / (SCAN_BLOCK * SCAN_ITEMS) + 2;
 #define TRY(x) do { e = (x); if (e != cudaSuccess) goto done; } while (0)
-    TRY(cudaMallocAsync(&off, sizeof(int64_t) * (nmax + 1), st));
-    TRY(cudaMallocAsync(&offb, sizeof(int64_t) * (N + 1), st));
-    TRY(cudaMallocAsync(&scratch, sizeof(int64_t) * nsb, st));
-    TRY(cudaMallocAsync(&total, sizeof(int64_t) * 2, st));
-    TRY(cudaMallocAsync(&key, sizeof(int64_t) * (S > 0 ? S : 1), st));
-    TRY(cudaMallocAsync(&bidx, sizeof(int64_t) * (F + 1), st));
-    TRY(cudaMallocAsync(&fill, sizeof(int32_t) * (N + 1), st));
-    TRY(cudaMallocAsync(&isp, sizeof(int32_t) * (N + 1), st));
-    TRY(cudaMallocAsync(&isb, sizeof(int32_t) * (nmax), st));
-    TRY(cudaMallocAsync(&maxrow, sizeof(int), st));
+    TRY(dev_alloc(&off, sizeof(int64_t) * (nmax + 1)));
+    TRY(dev_alloc(&offb, sizeof(int64_t) * (N + 1)));
+    TRY(dev_alloc(&scratch, sizeof(int64_t) * nsb));
+    TRY(dev_alloc(&total, sizeof(int64_t) * 2));
+    TRY(dev_alloc(&key, sizeof(int64_t) * (S > 0 ? S : 1)));
+    TRY(dev_alloc(&bidx, sizeof(int64_t) * (F + 1)));
+    TRY(dev_alloc(&fill, sizeof(int32_t) * (N + 1)));
+    TRY(dev_alloc(&isp, sizeof(int32_t) * (N + 1)));
+    TRY(dev_alloc(&isb, sizeof(int32_t) * (nmax)));
+    TRY(dev_alloc(&maxrow, sizeof(int)));
     TRY(cudaMemsetAsync(d_tmp, 0, sizeof(int32_t) * (N + 1), st));
     TRY(cudaMemsetAsync(fill, 0, sizeof(int32_t) * (N + 1), st));
     TRY(cudaMemsetAsync(maxrow, 0, sizeof(int), st));
@@ -332,27 +332,27 @@ cudaError_t launch_build_csr(const DevMesh& mc, const int32_t* fc, const double*
         m.n_pcells = N > 0 ? tot[0] : 0;
         m.n_bcells = N > 0 ? tot[1] : 0;
         if (m.n_pcells > 0) {
-            TRY(cudaMalloc(&m.pcells, sizeof(int32_t) * m.n_pcells));
+            TRY(dev_alloc(&m.pcells, sizeof(int32_t) * m.n_pcells));
             k_compact<<<nblk(N), 256, 0, st>>>(N, isp, off, m.pcells);
         }
         if (m.n_bcells > 0) {
-            TRY(cudaMalloc(&m.bcells, sizeof(int32_t) * m.n_bcells));
+            TRY(dev_alloc(&m.bcells, sizeof(int32_t) * m.n_bcells));
             k_compact<<<nblk(N), 256, 0, st>>>(N, isb, offb, m.bcells);
         }
         TRY(cudaGetLastError());
         TRY(cudaStreamSynchronize(st));
     }
 done:
-    cudaFreeAsync(off, st);
-    cudaFreeAsync(offb, st);
-    cudaFreeAsync(scratch, st);
-    cudaFreeAsync(total, st);
-    cudaFreeAsync(key, st);
-    cudaFreeAsync(bidx, st);
-    cudaFreeAsync(fill, st);
-    cudaFreeAsync(isp, st);
-    cudaFreeAsync(isb, st);
-    cudaFreeAsync(maxrow, st);
+    dev_free(off);
+    dev_free(offb);
+    dev_free(scratch);
+    dev_free(total);
+    dev_free(key);
+    dev_free(bidx);
+    dev_free(fill);
+    dev_free(isp);
+    dev_free(isb);
+    dev_free(maxrow);
 #undef TRY
     return e;
 }
@@ -1366,18 +1366,18 @@ cudaError_t pack_plan(const DevMesh& m, const Levels& L, PackedOp& P, bool trans
     if (want > P.grp_cap || !P.flag) {
         for (void* p : {(void*)P.grp, (void*)P.lev_grp, (void*)P.cnt, (void*)P.off, (void*)P.scan, (void*)P.lev_pk,
                         (void*)P.flag})
-            if (p) cudaFree(p);
+            if (p) dev_free(p);
         P.grp = nullptr; P.lev_grp = nullptr; P.cnt = nullptr; P.off = nullptr; P.scan = nullptr;
         P.lev_pk = nullptr; P.flag = nullptr;
         P.grp_cap = 0;
         const int64_t cap = want + want / 4;
-        if ((e = cudaMalloc(&P.grp, sizeof(int2) * cap))) return e;
-        if ((e = cudaMalloc(&P.lev_grp, sizeof(int32_t) * cap))) return e;
-        if ((e = cudaMalloc(&P.cnt, sizeof(int32_t) * cap))) return e;
-        if ((e = cudaMalloc(&P.off, sizeof(int64_t) * cap))) return e;
-        if ((e = cudaMalloc(&P.scan, sizeof(int64_t) * (cap / (SCAN_BLOCK * SCAN_ITEMS) + 2)))) return e;
-        if ((e = cudaMalloc(&P.lev_pk, sizeof(int64_t) * cap))) return e;
-        if ((e = cudaMalloc(&P.flag, sizeof(int32_t)))) return e;
+        if ((e = dev_alloc(&P.grp, sizeof(int2) * cap))) return e;
+        if ((e = dev_alloc(&P.lev_grp, sizeof(int32_t) * cap))) return e;
+        if ((e = dev_alloc(&P.cnt, sizeof(int32_t) * cap))) return e;
+        if ((e = dev_alloc(&P.off, sizeof(int64_t) * cap))) return e;
+        if ((e = dev_alloc(&P.scan, sizeof(int64_t) * (cap / (SCAN_BLOCK * SCAN_ITEMS) + 2)))) return e;
+        if ((e = dev_alloc(&P.lev_pk, sizeof(int64_t) * cap))) return e;
+        if ((e = dev_alloc(&P.flag, sizeof(int32_t)))) return e;
         P.grp_cap = cap;
     }
     P.ng = ng;
@@ -1434,11 +1434,11 @@ cudaError_t classify(const DevMesh& m, Levels& L, const float4* om32, const floa
 cudaError_t ensure_seg(Levels& L, int nlev) {
     const int nd = L.nd;
     if ((int64_t)nlev * (nd + 1) <= L.seg_cap) return cudaSuccess;
-    if (L.seg_off) cudaFree(L.seg_off);
+    if (L.seg_off) dev_free(L.seg_off);
     L.seg_off = nullptr;
     L.seg_cap = 0;
     const int64_t want = ((int64_t)nlev + nlev / 4 + 16) * (nd + 1);
-    cudaError_t e = cudaMalloc(&L.seg_off, sizeof(uint32_t) * want);
+    cudaError_t e = dev_alloc(&L.seg_off, sizeof(uint32_t) * want);
     if (e != cudaSuccess) return e;
     L.seg_cap = want;
     return cudaSuccess;
@@ -1447,8 +1447,8 @@ cudaError_t ensure_seg(Levels& L, int nlev) {
 // Device memory for the level-major task list.
 cudaError_t alloc_merged(Levels& L) {
     cudaError_t e = cudaSuccess;
-    if (!L.task) e = cudaMalloc(&L.task, sizeof(uint32_t) * L.task_cap);
-    if (e == cudaSuccess && !L.trec) e = cudaMalloc(&L.trec, sizeof(int4) * L.task_cap);
+    if (!L.task) e = dev_alloc(&L.task, sizeof(uint32_t) * L.task_cap);
+    if (e == cudaSuccess && !L.trec) e = dev_alloc(&L.trec, sizeof(int4) * L.task_cap);
     return e;
 }
 
@@ -1502,7 +1502,7 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
     if (L.n_levels == 0 || *done != m.N * (int64_t)nd) return cudaSuccess;
     // the cells of each (direction, level) in cell order
     if (!L.lfill) {
-        if ((e = cudaMalloc(&L.lfill, sizeof(int32_t) * (size_t)nd * cap))) return e;
+        if ((e = dev_alloc(&L.lfill, sizeof(int32_t) * (size_t)nd * cap))) return e;
     }
     if ((e = cudaMemsetAsync(L.lfill, 0, sizeof(int32_t) * (size_t)nd * cap, st))) return e;
     const int64_t tot = m.N * (int64_t)nd;

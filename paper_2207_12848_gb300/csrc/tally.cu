@@ -581,10 +581,10 @@ cudaError_t build_periodic_table(const DevMesh& m, int nd, const double* om64, c
     const int64_t np = m.n_pcells;
     cudaError_t e;
     if (t->off_cap < (size_t)(2 * (np + 1))) {
-        if (t->off) cudaFree(t->off);
+        if (t->off) dev_free(t->off);
         t->off = nullptr;
         t->off_cap = 0;
-        if ((e = cudaMalloc(&t->off, sizeof(int32_t) * 2 * (np + 1)))) return e;
+        if ((e = dev_alloc(&t->off, sizeof(int32_t) * 2 * (np + 1)))) return e;
         t->off_cap = 2 * (np + 1);
     }
     int32_t* cnt = t->off + (np + 1);
@@ -595,10 +595,10 @@ cudaError_t build_periodic_table(const DevMesh& m, int nd, const double* om64, c
     if ((e = cudaStreamSynchronize(st))) return e;
     const size_t need = (size_t)(total > 0 ? total : 1) * nd;
     if (t->wa_cap < need) {
-        if (t->wa) cudaFree(t->wa);
+        if (t->wa) dev_free(t->wa);
         t->wa = nullptr;
         t->wa_cap = 0;
-        if ((e = cudaMalloc(&t->wa, sizeof(double) * need))) return e;
+        if ((e = dev_alloc(&t->wa, sizeof(double) * need))) return e;
         t->wa_cap = need;
     }
     k_pside_weights<<<(unsigned)np, ROW_THREADS, 0, st>>>(m.pcells, t->off, m.rowptr, m.side, m.side64, nd, om64, w64,
