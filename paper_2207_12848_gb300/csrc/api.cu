@@ -534,10 +534,8 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
             double* jr = (t & 1) ? jB : jA;  // j of the previous iteration
             double* jw = (t & 1) ? jA : jB;
             if ((e = cudaMemsetAsync(c->dmax, 0, sizeof(unsigned long long), gs))) return e;
-            if ((e = launch_periodic_source(prec, c->mesh, b.I[cur], G, D, c->om64, c->w64, jw, jr, c->dmax,
-                                            c->partial, nblk, gs, &c->ptab)))
-                return e;
-            if ((e = launch_reduce_sum(c->partial, (int)c->mesh.n_pcells, c->red + 2, gs))) return e;
+            if ((e = launch_periodic_source(prec, c->mesh, b.I[cur], G, D, jw, jr, c->partial, gs, c->ptab))) return e;
+            if ((e = launch_reduce_change(c->partial, (int)c->mesh.n_pcells, c->red + 2, c->dmax, gs))) return e;
             if ((e = cudaMemcpyAsync(hp->red, c->red + 2, 2 * sizeof(double), cudaMemcpyDeviceToHost, gs))) return e;
         }
         if ((e = cudaEventRecordWithFlags(ev[2], gs, cudaEventRecordExternal))) return e;
@@ -686,7 +684,7 @@ sweep_status sweep_destroy(sweep_ctx* c) {
     dfree(c->J); dfree(c->Jold); dfree(c->Gam); dfree(c->jn); dfree(c->jn1);
     dfree(c->partial); dfree(c->red); dfree(c->dmax); dfree(c->bar); dfree(c->derr); dfree(c->scratch);
     dfree(c->stall_word);
-    dfree(c->ptab.off); dfree(c->ptab.wa);
+    dfree(c->ptab.off); dfree(c->ptab.wa); dfree(c->ptab.partner); dfree(c->ptab.rec);
     if (c->gst) cudaStreamDestroy(c->gst);
     if (c->hpin) cudaFreeHost(c->hpin);
     delete c;
@@ -1332,7 +1330,6 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     // the periodic inflow of the first sweep: the previous solve's intensities or zeros
     int prev = -1;
     if (has_pbc) {
-        c->ptab.ready = false;
         const DcTabs dct = dc_tabs(c, c->lev);
         CK(build_periodic_table(c->mesh, D, c->om64, c->w64, &c->ptab, c->st, &dct), "periodic weights");
         c->launches += 3;
@@ -1344,9 +1341,8 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         }
         CK(cudaMemsetAsync(c->jn, 0, sizeof(double) * NG, c->st), "init");
         if (o.warm_start && b.last >= 0) {
-            CK(cudaMemsetAsync(c->dmax, 0, sizeof(unsigned long long), c->st), "init");
-            CKL(launch_periodic_source(prec, c->mesh, b.I[prev], G, D, c->om64, c->w64, c->jn1, c->jn, c->dmax,
-                                      c->partial, nblk, c->st, &c->ptab), "periodic source");
+            CKL(launch_periodic_source(prec, c->mesh, b.I[prev], G, D, c->jn1, c->jn, c->partial, c->st, c->ptab),
+                "periodic source");
             std::swap(c->jn, c->jn1);
         }
     }
@@ -1434,9 +1430,9 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         if (!has_pbc) break;
         cudaEventRecord(u0, c->st);
         CK(cudaMemsetAsync(c->dmax, 0, sizeof(unsigned long long), c->st), "init");
-        CKL(launch_periodic_source(prec, c->mesh, b.I[cur], G, D, c->om64, c->w64, c->jn1, c->jn, c->dmax, c->partial,
-                                  nblk, c->st, &c->ptab), "periodic source");
-        CKL(launch_reduce_sum(c->partial, (int)c->mesh.n_pcells, c->red + 2, c->st), "reduce");
+        CKL(launch_periodic_source(prec, c->mesh, b.I[cur], G, D, c->jn1, c->jn, c->partial, c->st, c->ptab),
+            "periodic source");
+        CKL(launch_reduce_change(c->partial, (int)c->mesh.n_pcells, c->red + 2, c->dmax, c->st), "reduce");
         cudaEventRecord(u1, c->st);
         res_pbc = read_max(c);
         double hred[2] = {0, 0};

@@ -606,14 +606,17 @@ struct PeriodicTable {
     size_t off_cap = 0;
     double* wa = nullptr;     // [periodic sides][nd] w_d A |n.Omega| on inflow sides, else 0
     size_t wa_cap = 0;
-    bool ready = false;
+    int32_t* partner = nullptr;  // [periodic sides] partner cell
+    size_t partner_cap = 0;
+    int4* rec = nullptr;         // [n_pcells] cell, first and end of its periodic sides
+    size_t rec_cap = 0;
 };
 cudaError_t build_periodic_table(const DevMesh& m, int nd, const double* om64, const double* w64, PeriodicTable* t,
                                  cudaStream_t st, const DcTabs* dc = nullptr);
-cudaError_t launch_periodic_source(int precision, const DevMesh& m, const void* I, int G, int nd,
-                                   const double* om64, const double* w64, double* jn1, const double* jn,
-                                   unsigned long long* d_max, double* partial, int nblk, cudaStream_t st,
-                                   const PeriodicTable* tab = nullptr);
+cudaError_t launch_periodic_source(int precision, const DevMesh& m, const void* I, int G, int nd, double* jn1,
+                                   const double* jn, double* partial, cudaStream_t st, const PeriodicTable& tab);
+// sum and largest of the relative changes that launch_periodic_source left in partial
+cudaError_t launch_reduce_change(const double* partial, int n, double* out, unsigned long long* d_max, cudaStream_t st);
 cudaError_t launch_reduce_sum(const double* partial, int n, double* out, cudaStream_t st);
 cudaError_t launch_grad_accum(int precision, const void* I, const void* lam, int64_t N, int G, int nd, int d0,
                               const double* w64, const double* vol, const double* dl_dG, double* gk, double* ge,
