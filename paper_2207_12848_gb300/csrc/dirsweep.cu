@@ -985,7 +985,10 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         L.dir_ws = nullptr;
         L.dir_ws_bytes = 0;
         if (off + ((size_t)2 << 30) > dev_available()) return cudaSuccess;
-        if ((e = dev_alloc(&L.dir_ws, off))) return e;
+        if (dev_alloc(&L.dir_ws, off) != cudaSuccess) {  // no room: the packets take their place
+            cudaGetLastError();
+            return cudaSuccess;
+        }
         L.dir_ws_bytes = off;
     }
     const size_t keep = ((sizeof(DirMeta) * nd + 255) & ~(size_t)255) + 8 * nR;
@@ -993,7 +996,10 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         if (P.meta) dev_free(P.meta);
         P.meta = nullptr;
         P.meta_bytes = 0;
-        if ((e = dev_alloc(&P.meta, keep))) return e;
+        if (dev_alloc(&P.meta, keep) != cudaSuccess) {
+            cudaGetLastError();
+            return cudaSuccess;
+        }
         P.meta_bytes = keep;
     }
     P.rtab = (uint2*)((char*)P.meta + ((sizeof(DirMeta) * nd + 255) & ~(size_t)255));
