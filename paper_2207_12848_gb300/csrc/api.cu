@@ -134,7 +134,7 @@ void free_levels(Levels& L) {
 }
 
 void free_mesh(DevMesh& m) {
-    dfree(m.rowptr); dfree(m.side); dfree(m.side64); dfree(m.side_lo); dfree(m.ids); dfree(m.twin); dfree(m.vol);
+    dfree(m.rowptr); dfree(m.side); dfree(m.side64); dfree(m.ids); dfree(m.twin); dfree(m.vol);
     dfree(m.pcells); dfree(m.bcells);
     m = DevMesh();
 }
@@ -326,7 +326,6 @@ SweepArgs make_args(sweep_ctx* c, const Levels& L, int precision, const void* cm
     a.rowptr = c->mesh.rowptr;
     a.side = c->mesh.side;
     a.side64 = c->mesh.side64;
-    a.side_lo = c->mesh.side_lo;
     a.om32 = c->om32 + L.d0;
     a.om32lo = c->om32lo + L.d0;
     a.om64 = c->om64 + 3 * (int64_t)L.d0;
@@ -773,9 +772,8 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     m.vol = d_vol;
     m.mesh_off = off;
     CKM(dev_alloc(&m.rowptr, sizeof(uint32_t) * (n_cells + 1)), "alloc rows");
-    CKM(dev_alloc(&m.side, sizeof(int4) * (S > 0 ? S : 1) + 64 * sizeof(int4)), "alloc sides");
+    CKM(dev_alloc(&m.side, sizeof(SideRec) * ((S > 0 ? S : 1) + 64)), "alloc sides");
     CKM(dev_alloc(&m.side64, sizeof(d4) * (S > 0 ? S : 1)), "alloc sides");
-    CKM(dev_alloc(&m.side_lo, sizeof(float4) * (S > 0 ? S : 1)), "alloc sides");
     CKM(dev_alloc(&m.ids, sizeof(int32_t) * 32 * n_cells), "alloc sides");
     CKM(dev_alloc(&m.twin, sizeof(uint32_t) * (S > 0 ? S : 1)), "alloc sides");
     CKM(launch_build_csr(m, d_fc, d_area, d_normal, d_flags, d_tmp, c->st), "build CSR");

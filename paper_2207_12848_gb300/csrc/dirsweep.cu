@@ -96,9 +96,8 @@ struct DirBuild {
     int32_t* stat;             // [0] does not apply, [1] most far sources of a slice, [2] most C bytes, [3] most E bytes
     unsigned char *E, *C;
     const uint32_t* rowptr;
-    const int4* side;
+    const SideRec* side;
     const d4* side64;
-    const float4* side_lo;
     const float4 *om32, *om32lo;
     const double* om64;
     const int4* info;
@@ -120,7 +119,7 @@ __device__ uint64_t entry_mask(const DirBuild& a, uint32_t c, int d, float* P) {
     const double* o64 = a.om64 + 3 * d;
     uint64_t m = a.transposed ? 0ull : (uint32_t)info.z;
     for (uint32_t s = a.transposed ? r0 : r0 + 32; s < r1; ++s) {
-        const int4 r = a.side[s];
+        const int4 r = a.side[s].hi;
         if (a.transposed && r.x < 0) continue;
         const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
         const int sg = classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, o64);
@@ -301,7 +300,7 @@ __global__ void __launch_bounds__(128) k_dir_count(DirBuild a) {
         if (m) {
             const uint32_t r0 = a.rowptr[a.ord[t]];
             for (; m; m &= m - 1)
-                far += near_slot(a, d, a.side[r0 + (uint32_t)(__ffsll((long long)m) - 1)].x, end) == ~0u;
+                far += near_slot(a, d, a.side[r0 + (uint32_t)(__ffsll((long long)m) - 1)].hi.x, end) == ~0u;
         }
         far = __reduce_add_sync(0xffffffffu, far);
         if (lane == 0) {
@@ -401,7 +400,7 @@ __device__ __forceinline__ real entry_weight(const DirBuild& a, int d, uint32_t 
         const d4 n = a.side64[s];
         return (real)__dmul_rn(n.w, fabs(exact_t(n, a.om64 + 3 * d)));
     }
-    return (real)side_weight(r, a.side_lo[s], om, oml);
+    return (real)side_weight(r, a.side[s].lo, om, oml);
 }
 
 // Writes E and C: one block per round of a direction, a warp per slice.
@@ -460,7 +459,7 @@ __global__ void __launch_bounds__(128) k_dir_write(DirBuild a) {
                 const int b = 63 - __clzll((long long)left);
                 left &= ~(1ull << b);
                 const uint32_t s = r0 + (uint32_t)b;
-                const int4 sd = a.side[s];
+                const int4 sd = a.side[s].hi;
                 w[j] = entry_weight<real>(a, d, s, sd, om, oml);
                 const uint32_t slot = near_slot(a, d, sd.x, end);
                 if (slot != ~0u) {
@@ -1013,7 +1012,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     a.rinfo = (uint2*)(ws + o_ri); a.nfar = (uint32_t*)(ws + o_nf); a.coff = (uint32_t*)(ws + o_co); a.rtab = P.rtab;
     a.tot = (int2*)(ws + o_to); a.meta = P.meta; a.stat = (int32_t*)(ws + o_st);
     a.E = nullptr; a.C = nullptr;
-    a.rowptr = m.rowptr; a.side = m.side; a.side64 = m.side64; a.side_lo = m.side_lo;
+    a.rowptr = m.rowptr; a.side = m.side; a.side64 = m.side64;
     a.om32 = om32_all + L.d0; a.om32lo = om32lo_all + L.d0; a.om64 = om64_all + 3 * (int64_t)L.d0;
     a.info = L.info;
     const bool dc = L.transport > 0 && !transposed;

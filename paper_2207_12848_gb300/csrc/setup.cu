@@ -184,7 +184,7 @@ __global__ void k_flag_boundary(int64_t F, const uint8_t* flags, int32_t* isb) {
 
 __global__ void k_fill_sides(int64_t S, const int64_t* key, const int32_t* fc, const double* area,
                              const double* normal, const uint8_t* flags, const int64_t* bidx,
-                             int4* side, d4* side64, float4* side_lo) {
+                             SideRec* side, d4* side64) {
     int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (s >= S) return;
     int64_t k = key[s];
@@ -208,19 +208,18 @@ __global__ void k_fill_sides(int64_t S, const int64_t* key, const int32_t* fc, c
     r.y = __float_as_int(hx);
     r.z = __float_as_int(hy);
     r.w = __float_as_int(hz);
-    side[s] = r;
     side64[s] = d4{nx, ny, nz, A};
-    side_lo[s] = make_float4((float)(ax - (double)hx), (float)(ay - (double)hy), (float)(az - (double)hz), 0.f);
+    side[s] = SideRec{r, make_float4((float)(ax - (double)hx), (float)(ay - (double)hy), (float)(az - (double)hz), 0.f)};
 }
 
 // Neighbour codes of each cell's first 32 sides at a fixed place (-1 past the row's end): the levelisation reads
 // them without the row bounds, 4 bytes a side.
-__global__ void k_fill_ids(int64_t N, const uint32_t* rowptr, const int4* side, int32_t* ids) {
+__global__ void k_fill_ids(int64_t N, const uint32_t* rowptr, const SideRec* side, int32_t* ids) {
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (t >= N * 32) return;
     const int64_t c = t >> 5;
     const uint32_t s = rowptr[c] + (uint32_t)(t & 31);
-    ids[t] = s < rowptr[c + 1] ? side[s].x : -1;
+    ids[t] = s < rowptr[c + 1] ? side[s].hi.x : -1;
 }
 
 // Position of each interior or periodic side's twin (the same face seen from the neighbour) in the
@@ -246,12 +245,12 @@ __global__ void k_twin(int64_t S, const int64_t* key, const int32_t* fc, const u
     twin[s] = lo - rowptr[u];
 }
 
-__global__ void k_cell_kinds(int64_t N, const uint32_t* rowptr, const int4* side, int32_t* isp, int32_t* isb) {
+__global__ void k_cell_kinds(int64_t N, const uint32_t* rowptr, const SideRec* side, int32_t* isp, int32_t* isb) {
     int64_t c = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (c >= N) return;
     int p = 0, b = 0;
     for (uint32_t s = rowptr[c]; s < rowptr[c + 1]; ++s) {
-        int32_t nb = side[s].x;
+        int32_t nb = side[s].hi.x;
         if (nb < 0) b = 1;
         else if (nb & NBR_PERIODIC) p = 1;
     }
@@ -312,8 +311,7 @@ cudaError_t launch_build_csr(const DevMesh& mc, const int32_t* fc, const double*
         k_flag_boundary<<<nblk(F), 256, 0, st>>>(F, flags, isb);
         TRY(scan_i32(isb, F, bidx, scratch, total, st));
     }
-    if (S > 0) k_fill_sides<<<nblk(S), 256, 0, st>>>(S, key, fc, area, normal, flags, bidx, m.side, m.side64,
-                                                     m.side_lo);
+    if (S > 0) k_fill_sides<<<nblk(S), 256, 0, st>>>(S, key, fc, area, normal, flags, bidx, m.side, m.side64);
     if (N > 0) k_fill_ids<<<nblk(N * 32), 256, 0, st>>>(N, m.rowptr, m.side, m.ids);
     if (S > 0) k_twin<<<nblk(S), 256, 0, st>>>(S, key, fc, flags, m.rowptr, m.twin);
     // periodic / boundary cell lists (increasing cell order)
@@ -368,8 +366,8 @@ namespace {
 //               P_c: FP32 projected outflow area (sign bit set when the row has more than 32 sides),
 //               bit k: side k (< 32) is an inflow side (any kind),
 //               bit k: side k (< 32) is an outflow side to an interior cell}
-__global__ void k_classify(int64_t N, int nd, const uint32_t* rowptr, const int4* side, const d4* side64,
-                           const float4* side_lo, const float4* om32, const float4* om32lo, const double* om64,
+__global__ void k_classify(int64_t N, int nd, const uint32_t* rowptr, const SideRec* side, const d4* side64,
+                           const float4* om32, const float4* om32lo, const double* om64,
                            int4* info, int32_t* level, uint32_t* raw, int32_t* lvl_cnt, int cshift, uint32_t* dlist,
                            int32_t* n0, unsigned long long* word) {
     int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -385,14 +383,14 @@ __global__ void k_classify(int64_t N, int nd, const uint32_t* rowptr, const int4
         float P = 0.f;
         uint32_t inm = 0u, outm = 0u;
         for (uint32_t s = r0; s < r1; ++s) {
-            int4 r = side[s];
+            int4 r = side[s].hi;
             float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
             const int sgn = classify_side(dot32(ax, ay, az, om), ax, ay, az, side64, s, o64);
             if (sgn == 0) continue;
             const uint32_t k = s - r0;
             const bool interior = r.x >= 0 && !(r.x & NBR_PERIODIC);
             if (sgn > 0) {
-                P += side_weight(r, side_lo[s], om, oml);
+                P += side_weight(r, side[s].lo, om, oml);
                 if (k < 32 && interior) outm |= 1u << k;
             } else {
                 if (k < 32) inm |= 1u << k;
@@ -485,7 +483,7 @@ __global__ void k_dc_choose(int64_t N, int nd, int dcn, const uint32_t* rowptr, 
 // chose the face (read through the twin side's position in the upwind row), and boundary inflow sides,
 // which enter as in scheme (a) -- and the upwind count over the chosen interior faces, which seeds the
 // levelisation (its words: chosen sides and count; level-0 lists per direction).
-__global__ void k_dc_count(int64_t N, int nd, const uint32_t* rowptr, const int4* side, const d4* side64,
+__global__ void k_dc_count(int64_t N, int nd, const uint32_t* rowptr, const SideRec* side, const d4* side64,
                            const float4* om32, const double* om64, const uint32_t* twin, const uint64_t* dc_mask,
                            uint64_t* dc_inm, int32_t* level, uint32_t* dlist, int32_t* n0,
                            unsigned long long* word) {
@@ -499,7 +497,7 @@ __global__ void k_dc_count(int64_t N, int nd, const uint32_t* rowptr, const int4
     uint64_t inm = 0ull;
     int cnt = 0;
     for (uint32_t s = r0; s < r1; ++s) {
-        const int4 r = side[s];
+        const int4 r = side[s].hi;
         const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
         if (classify_side(dot32(ax, ay, az, om), ax, ay, az, side64, s, o64) >= 0) continue;
         const uint64_t bit = 1ull << (s - r0);
@@ -534,7 +532,7 @@ struct LeveliseArgs {
     int cshift;
     uint32_t cmask;
     const uint32_t* rowptr;
-    const int4* side;
+    const SideRec* side;
     const d4* side64;
     const float4* om32;
     const double* om64;
@@ -594,7 +592,7 @@ __global__ void __launch_bounds__(256) k_levelise(LeveliseArgs a) {
                         const uint32_t s = b + gl + k * KL;
                         const uint32_t idx = s - r0;
                         const bool need = s < r1 && (idx >= 32u || ((outm >> idx) & 1u));
-                        r[k] = need ? a.side[s] : make_int4(-1, 0, 0, 0);
+                        r[k] = need ? a.side[s].hi : make_int4(-1, 0, 0, 0);
                     }
                     int old[KU];
 #pragma unroll
@@ -703,7 +701,7 @@ struct DirLevArgs {
     int long_rows;           // some row has more than 32 sides
     const uint32_t* rowptr;
     const int32_t* ids;      // [N][32] neighbour codes of the first 32 sides
-    const int4* side;
+    const SideRec* side;
     const d4* side64;
     const float4* om32;
     const double* om64;
@@ -815,7 +813,7 @@ __global__ void __launch_bounds__(LD_THREADS, 1) k_levelise_dir(DirLevArgs a) {
                         int32_t x[LD_KU] = {};
                         unsigned long long o[LD_KU] = {};
                         if (s < r1) {
-                            const int4 r = a.side[s];
+                            const int4 r = a.side[s].hi;
                             const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
                             const bool go = r.x >= 0 && !(r.x & NBR_PERIODIC) &&
                                             (a.dc_mask ? (chosen >> (s - r0)) & 1ull
@@ -960,8 +958,8 @@ __global__ void k_gather_levels(const uint32_t* dlist, const int32_t* dcnt, cons
 //                Unused entries are {0, 0}.
 // One task's line built by one thread: rows longer than 32 sides (inflow mask plus classification of
 // the sides past 32), and the reference form of the assembly.
-__device__ void build_line_serial(const int4 tr, int4* line, const uint32_t* rowptr, const int4* side, const d4* side64,
-                                  const float4* side_lo, const float4* om32, const float4* om32lo, const double* om64,
+__device__ void build_line_serial(const int4 tr, int4* line, const uint32_t* rowptr, const SideRec* side, const d4* side64,
+                                  const float4* om32, const float4* om32lo, const double* om64,
                                   uint32_t cmask, int cshift, uint32_t N) {
     int2* E = reinterpret_cast<int2*>(line + 1);
     const uint32_t c = (uint32_t)tr.x & cmask, dl = (uint32_t)tr.x >> cshift;
@@ -973,7 +971,7 @@ __device__ void build_line_serial(const int4 tr, int4* line, const uint32_t* row
     uint32_t bmask = 0;
     auto put = [&](const int4& r, uint32_t s) {
         if (nin < OP_MAX) {
-            const float w = side_weight(r, side_lo[s], om, oml);
+            const float w = side_weight(r, side[s].lo, om, oml);
             int2 v;
             if (r.x >= 0 && !(r.x & NBR_PERIODIC)) {
                 v = make_int2((int)(slab + (uint32_t)r.x), __float_as_int(w));
@@ -989,12 +987,12 @@ __device__ void build_line_serial(const int4 tr, int4* line, const uint32_t* row
     };
     for (uint32_t m = (uint32_t)tr.w; m; m &= m - 1) {
         const uint32_t s = r0 + (uint32_t)(__ffs(m) - 1);
-        put(side[s], s);
+        put(side[s].hi, s);
     }
     if (tr.z < 0) {  // rows longer than 32 sides
         const uint32_t r1 = rowptr[c + 1];
         for (uint32_t s = r0 + 32; s < r1; ++s) {
-            const int4 r = side[s];
+            const int4 r = side[s].hi;
             const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
             if (classify_side(dot32(ax, ay, az, om), ax, ay, az, side64, s, o64) >= 0) continue;
             put(r, s);
@@ -1007,8 +1005,8 @@ __device__ void build_line_serial(const int4 tr, int4* line, const uint32_t* row
 // 8 lanes per task: lane 0 writes the header, lane g >= 1 the entries 2g-2 and 2g-1 (the (2g-2)-th and
 // (2g-1)-th inflow sides of the row in row order), so the side loads of a row run in parallel and the
 // 128-byte line is one coalesced store of the group. Rows longer than 32 sides take the serial form.
-__global__ void __launch_bounds__(256) k_build_op(const int4* trec, int64_t n, const uint32_t* rowptr, const int4* side,
-                                                  const d4* side64, const float4* side_lo, const float4* om32,
+__global__ void __launch_bounds__(256) k_build_op(const int4* trec, int64_t n, const uint32_t* rowptr, const SideRec* side,
+                                                  const d4* side64, const float4* om32,
                                                   const float4* om32lo, const double* om64, uint32_t cmask, int cshift,
                                                   uint32_t N, int4* op) {
     const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 3;  // task
@@ -1022,7 +1020,7 @@ __global__ void __launch_bounds__(256) k_build_op(const int4* trec, int64_t n, c
         return;
     }
     if (tr.z < 0) {
-        if (gl == 0) build_line_serial(tr, line, rowptr, side, side64, side_lo, om32, om32lo, om64, cmask, cshift, N);
+        if (gl == 0) build_line_serial(tr, line, rowptr, side, side64, om32, om32lo, om64, cmask, cshift, N);
         return;
     }
     const uint32_t c = (uint32_t)tr.x & cmask, dl = (uint32_t)tr.x >> cshift;
@@ -1041,8 +1039,8 @@ __global__ void __launch_bounds__(256) k_build_op(const int4* trec, int64_t n, c
             uint32_t m = inm;
             for (int q = 0; q < j; ++q) m &= m - 1;  // the j-th inflow side
             const uint32_t s = r0 + (uint32_t)(__ffs(m) - 1);
-            const int4 r = side[s];
-            const float w = side_weight(r, side_lo[s], om, oml);
+            const int4 r = side[s].hi;
+            const float w = side_weight(r, side[s].lo, om, oml);
             if (r.x >= 0 && !(r.x & NBR_PERIODIC)) {
                 ent[k] = make_int2((int)(slab + (uint32_t)r.x), __float_as_int(w));
             } else if (r.x >= 0) {
@@ -1066,7 +1064,7 @@ cudaError_t build_operator(const DevMesh& m, const Levels& L, const double* om64
                            const float4* om32lo_all, cudaStream_t st) {
     const int64_t n = L.h_lev_chunk.empty() ? 0 : L.h_lev_chunk.back() * 32;
     if (n > 0)
-        k_build_op<<<nblk(n * 8), 256, 0, st>>>(L.trec, n, m.rowptr, m.side, m.side64, m.side_lo, om32_all + L.d0,
+        k_build_op<<<nblk(n * 8), 256, 0, st>>>(L.trec, n, m.rowptr, m.side, m.side64, om32_all + L.d0,
                                             om32lo_all + L.d0, om64_all + 3 * (int64_t)L.d0, L.cmask, L.cshift,
                                             (uint32_t)m.N, L.op);
     return cudaGetLastError();
@@ -1103,9 +1101,8 @@ struct PackArgs {
     int64_t ng;
     int transposed;      // the adjoint's operator: outflow entries (interior and periodic sides)
     const uint32_t* rowptr;
-    const int4* side;
+    const SideRec* side;
     const d4* side64;
-    const float4* side_lo;
     const float4* om32;
     const float4* om32lo;
     const double* om64;
@@ -1130,7 +1127,7 @@ __device__ int pk_inflow_past32(const PackArgs& a, const int4 tr, int stop_at, u
     const uint32_t r0 = (uint32_t)tr.y, r1 = a.rowptr[c + 1];
     int k = 0;
     for (uint32_t s = r0 + 32; s < r1; ++s) {
-        const int4 r = a.side[s];
+        const int4 r = a.side[s].hi;
         const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
         if (classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, o64) >= 0) continue;
         if (k == stop_at) {
@@ -1151,7 +1148,7 @@ __device__ int pk_outflow(const PackArgs& a, const int4 tr, int stop_at, uint32_
     const uint32_t r0 = (uint32_t)tr.y, r1 = a.rowptr[c + 1];
     int k = 0;
     for (uint32_t s = r0; s < r1; ++s) {
-        const int4 r = a.side[s];
+        const int4 r = a.side[s].hi;
         if (r.x < 0) continue;  // boundary face: nothing flows back in through the transpose
         const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
         if (classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, o64) <= 0) continue;
@@ -1184,30 +1181,39 @@ __device__ __forceinline__ int pk_task_inflow(const PackArgs& a, const int4 tr) 
     return n;
 }
 
-__device__ __forceinline__ int nth_set_bit(uint32_t m, int j) {
-    for (int q = 0; q < j; ++q) m &= m - 1;
-    return __ffs(m) - 1;
-}
-
-// entry j of a task: its j-th inflow side in row order (scheme (b): of its effective inflow sides, the
-// interior and periodic ones weighted by the upwind cell's share)
-__device__ int2 pk_entry(const PackArgs& a, const int4 tr, int j, uint32_t slab, const float4& om, const float4& oml) {
-    uint32_t s = 0;
+// sides of entries j and (two) j + 1 of a task: its j-th inflow side in row order (scheme (b): of its effective inflow
+// sides)
+__device__ __forceinline__ void pk_sides(const PackArgs& a, const int4 tr, int j, bool two, uint32_t s[2]) {
+    s[0] = s[1] = (uint32_t)tr.y;
     if (a.transposed) {
-        pk_outflow(a, tr, j, &s);
+        pk_outflow(a, tr, j, &s[0]);
+        if (two) pk_outflow(a, tr, j + 1, &s[1]);
     } else if (a.dc_inm) {
         uint64_t m = a.dc_inm[pk_dc_index(a, (uint32_t)tr.x)];
         for (int q = 0; q < j; ++q) m &= m - 1;
-        s = (uint32_t)tr.y + (uint32_t)(__ffsll((long long)m) - 1);
+        s[0] = (uint32_t)tr.y + (uint32_t)(__ffsll((long long)m) - 1);
+        m &= m - 1;
+        if (two) s[1] = (uint32_t)tr.y + (uint32_t)(__ffsll((long long)m) - 1);
     } else {
-        const uint32_t inm = (uint32_t)tr.w;
-        const int nm = __popc(inm);
-        if (j < nm) s = (uint32_t)tr.y + (uint32_t)nth_set_bit(inm, j);
-        else pk_inflow_past32(a, tr, j - nm, &s);
+        uint32_t m = (uint32_t)tr.w;
+        const int nm = __popc(m);
+        for (int q = 0; q < j; ++q) m &= m - 1;
+        if (j < nm) s[0] = (uint32_t)tr.y + (uint32_t)(__ffs(m) - 1);
+        else pk_inflow_past32(a, tr, j - nm, &s[0]);
+        m &= m - 1;
+        if (two) {
+            if (j + 1 < nm) s[1] = (uint32_t)tr.y + (uint32_t)(__ffs(m) - 1);
+            else pk_inflow_past32(a, tr, j + 1 - nm, &s[1]);
+        }
     }
-    const int4 r = a.side[s];
-    float w = side_weight(r, a.side_lo[s], om, oml);
-    if (a.dc_inm && r.x >= 0) w = a.dc_share32[(int64_t)(r.x & NBR_MASK) * a.nd + ((uint32_t)tr.x >> a.cshift)];
+}
+
+// the slot of a side: {source, weight} (scheme (b): interior and periodic sides weighted by the upwind cell's share)
+__device__ __forceinline__ int2 pk_entry(const PackArgs& a, uint32_t e, const SideRec& sr, uint32_t slab, const float4& om,
+                                         const float4& oml) {
+    const int4 r = sr.hi;
+    float w = side_weight(r, sr.lo, om, oml);
+    if (a.dc_inm && r.x >= 0) w = a.dc_share32[(int64_t)(r.x & NBR_MASK) * a.nd + (e >> a.cshift)];
     if (r.x >= 0 && !(r.x & NBR_PERIODIC)) return make_int2((int)(slab + (uint32_t)r.x), __float_as_int(w));
     if (r.x >= 0) return make_int2((int)(slab + (uint32_t)(r.x & NBR_MASK)), __float_as_int(-w));
     return make_int2((int)((uint32_t)(-1 - r.x) | PK_BOUNDARY), __float_as_int(-w));
@@ -1241,9 +1247,15 @@ __global__ void __launch_bounds__(256) k_pack(PackArgs a) {
                 const uint32_t slab = dl * a.N;
                 const float4 om = a.om32[dl], oml = a.om32lo[dl];
                 const int j0 = 2 * my_j;
-                const int2 s0 = j0 < my_n ? pk_entry(a, my_tr, j0, slab, om, oml) : make_int2(0, 0);
-                const int2 s1 = head ? make_int2(my_tr.x, my_tr.z & 0x7fffffff)
-                                     : (j0 + 1 < my_n ? pk_entry(a, my_tr, j0 + 1, slab, om, oml) : make_int2(0, 0));
+                int2 s0 = make_int2(0, 0), s1 = head ? make_int2(my_tr.x, my_tr.z & 0x7fffffff) : make_int2(0, 0);
+                if (j0 < my_n) {
+                    const bool two = !head && j0 + 1 < my_n;
+                    uint32_t s[2];
+                    pk_sides(a, my_tr, j0, two, s);
+                    const SideRec ra = a.side[s[0]], rb = a.side[two ? s[1] : s[0]];  // both in flight
+                    s0 = pk_entry(a, (uint32_t)my_tr.x, ra, slab, om, oml);
+                    if (two) s1 = pk_entry(a, (uint32_t)my_tr.x, rb, slab, om, oml);
+                }
                 out = make_int4(s0.x, s0.y, s1.x, s1.y);
             }
             const unsigned hm = __ballot_sync(0xffffffffu, head);
@@ -1325,7 +1337,6 @@ PackArgs pack_args(const DevMesh& m, const Levels& L, const PackedOp& P, bool tr
     a.rowptr = m.rowptr;
     a.side = m.side;
     a.side64 = m.side64;
-    a.side_lo = m.side_lo;
     a.om32 = om32_all + L.d0;
     a.om32lo = om32lo_all + L.d0;
     a.om64 = om64_all + 3 * (int64_t)L.d0;
@@ -1425,7 +1436,7 @@ cudaError_t classify(const DevMesh& m, Levels& L, const float4* om32, const floa
     }
     const int64_t tot = N * (int64_t)nd;
     if (tot > 0)
-        k_classify<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, m.side_lo, om32, om32lo, om64,
+        k_classify<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, om32, om32lo, om64,
                                                L.info, L.level, L.raw, L.lvl_cnt, L.cshift,
                                                per_direction ? L.raw : nullptr, n0, L.word);
     return cudaGetLastError();

@@ -113,9 +113,9 @@ __device__ __noinline__ bool wait_value_slow(const real* p, int parity, const Sw
 constexpr int SLOTS = 16;
 // L2 prefetch of a task's face-side row by the bulk-copy engine (the row is contiguous, 16-byte
 // records, so address and size are multiples of 16 bytes)
-__device__ __forceinline__ void prefetch_row(const int4* side, uint32_t r0, uint32_t r1) {
+__device__ __forceinline__ void prefetch_row(const SideRec* side, uint32_t r0, uint32_t r1) {
     if (r1 > r0)
-        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(side + r0), "r"((r1 - r0) * 16u));
+        asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(side + r0), "r"((r1 - r0) * (unsigned)sizeof(SideRec)));
 }
 
 template <typename real, int GC, int L>
@@ -158,7 +158,7 @@ __device__ __forceinline__ bool group_task(const SweepArgs& a, uint32_t entry, u
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             const uint32_t s = base + gl + k * L;
-            rec[k] = s < r1 ? ld_stream_int4(a.side + s, pol) : make_int4(0, 0, 0, 0);
+            rec[k] = s < r1 ? ld_stream_int4(&a.side[s].hi, pol) : make_int4(0, 0, 0, 0);
         }
         real w[U];
         int kind[U];  // 0 none, 1 interior inflow, 2 periodic inflow (adjoint: its transpose), 3 boundary inflow
@@ -178,7 +178,7 @@ __device__ __forceinline__ bool group_task(const SweepArgs& a, uint32_t entry, u
                     const float ax = __int_as_float(rec[k].y), ay = __int_as_float(rec[k].z),
                                 az = __int_as_float(rec[k].w);
                     sgn = classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, om64);
-                    if (sgn != 0) w[k] = (real)side_weight(rec[k], a.side_lo[s], om, oml);
+                    if (sgn != 0) w[k] = (real)side_weight(rec[k], a.side[s].lo, om, oml);
                 }
                 if (sgn > 0) P = addr(P, w[k]);
                 const bool inflow = sgn != 0 && (a.reverse ? (sgn > 0) : (sgn < 0));
@@ -412,7 +412,7 @@ __device__ __forceinline__ bool rec_task(const SweepArgs& a, const int4 tr, cons
         }
         int4 rec[U];
 #pragma unroll
-        for (int k = 0; k < U; ++k) rec[k] = ok[k] ? ld_stream_int4(a.side + r0 + pos[k], pol) : make_int4(-1, 0, 0, 0);
+        for (int k = 0; k < U; ++k) rec[k] = ok[k] ? ld_stream_int4(&a.side[r0 + pos[k]].hi, pol) : make_int4(-1, 0, 0, 0);
         float v[U][GM];
 #pragma unroll
         for (int k = 0; k < U; ++k) {
@@ -426,7 +426,7 @@ __device__ __forceinline__ bool rec_task(const SweepArgs& a, const int4 tr, cons
 #pragma unroll
         for (int k = 0; k < U; ++k) {
             if (!ok[k]) continue;
-            const float w = side_weight(rec[k], __ldg(a.side_lo + r0 + pos[k]), om, oml);
+            const float w = side_weight(rec[k], __ldg(&a.side[r0 + pos[k]].lo), om, oml);
             add_inflow<GC>(a, rec[k].x, w, v[k], slab, G, acc, fail);
         }
     }
@@ -434,10 +434,10 @@ __device__ __forceinline__ bool rec_task(const SweepArgs& a, const int4 tr, cons
         const uint32_t r1 = __ldg(a.rowptr + c + 1);
         const double* om64 = a.om64 + 3 * dl;
         for (uint32_t s = r0 + 32 + gl; s < r1; s += L) {
-            const int4 r = a.side[s];
+            const int4 r = a.side[s].hi;
             const float ax = __int_as_float(r.y), ay = __int_as_float(r.z), az = __int_as_float(r.w);
             if (classify_side(dot32(ax, ay, az, om), ax, ay, az, a.side64, s, om64) < 0)
-                add_inflow<GC>(a, r.x, side_weight(r, a.side_lo[s], om, oml), nullptr, slab, G, acc, fail);
+                add_inflow<GC>(a, r.x, side_weight(r, a.side[s].lo, om, oml), nullptr, slab, G, acc, fail);
         }
     }
 #pragma unroll
@@ -463,7 +463,7 @@ __device__ __forceinline__ bool rec_task(const SweepArgs& a, const int4 tr, cons
 __device__ __forceinline__ void prefetch_rec(const SweepArgs& a, const int4 tr) {
     if ((uint32_t)tr.x == TASK_PAD || tr.w == 0) return;
     const uint32_t n = 32u - __clz((uint32_t)tr.w);
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.side + (uint32_t)tr.y), "r"(n * 16u));
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(a.side + (uint32_t)tr.y), "r"(n * (unsigned)sizeof(SideRec)));
 }
 
 template <int GC, int L, typename ChunkFn>
@@ -1340,7 +1340,7 @@ __device__ __forceinline__ void plain_task(const SweepArgs& a, uint32_t entry) {
         if (g < G) acc[g] = a.law ? 0.0 : (a.reverse ? __dmul_rn(a.w64[dl], cm[g].x) : cm[g].x);
     double P = 0.0;
     for (uint32_t s = r0; s < r1; ++s) {
-        const int32_t nb = a.side[s].x;
+        const int32_t nb = a.side[s].hi.x;
         const d4 n = a.side64[s];
         const double t = exact_t(n, om64);
         if (t == 0.0) continue;

@@ -180,7 +180,7 @@ __device__ __forceinline__ double block_sum_fixed(double v, double* sh) {
 // 110,000 boundary cells of 25 meshes, 128 directions, 2 groups.
 template <typename real>
 __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* bcells, const uint32_t* rowptr,
-                                                                const int4* side, const d4* side64, const real* I,
+                                                                const SideRec* side, const d4* side64, const real* I,
                                                                 int64_t N, int G, int nd, const double* om64,
                                                                 const double* w64, const double* bc,
                                                                 double* partial, DcTabs dc) {
@@ -194,7 +194,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* b
         const float fx = (float)ox, fy = (float)oy, fz = (float)oz;
         double out = 0.0;  // flux factor of the outflow through vacuum faces
         for (uint32_t s = r0; s < r1; ++s) {
-            const int4 rec = side[s];
+            const int4 rec = side[s].hi;
             if (rec.x >= 0) continue;
             if (!bc) {
                 const float ax = __int_as_float(rec.y), ay = __int_as_float(rec.z), az = __int_as_float(rec.w);
@@ -235,14 +235,14 @@ __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* b
 // instead of recomputing n.Omega and the weight on this part's narrow FP64 pipe. Beside the weights stand the
 // partner of each side and, per periodic cell, its number and its range of sides, so that an iteration reads
 // one record and consecutive lists instead of searching the cell's row for its periodic sides.
-__global__ void k_pside_count(const int32_t* pcells, int64_t np, const uint32_t* rowptr, const int4* side,
+__global__ void k_pside_count(const int32_t* pcells, int64_t np, const uint32_t* rowptr, const SideRec* side,
                               int32_t* cnt) {
     const int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= np) return;
     const int32_t c = pcells[k];
     int n = 0;
     for (uint32_t s = rowptr[c]; s < rowptr[c + 1]; ++s) {
-        const int32_t x = side[s].x;
+        const int32_t x = side[s].hi.x;
         if (x >= 0 && (x & NBR_PERIODIC)) ++n;
     }
     cnt[k] = n;
@@ -275,7 +275,7 @@ __global__ void k_scan_counts(const int32_t* cnt, int64_t n, int32_t* off) {
 }
 
 __global__ void __launch_bounds__(ROW_THREADS) k_pside_weights(const int32_t* pcells, const int32_t* off,
-                                                               const uint32_t* rowptr, const int4* side,
+                                                               const uint32_t* rowptr, const SideRec* side,
                                                                const d4* side64, int nd, const double* om64,
                                                                const double* w64, double* wa, int32_t* partner, int4* rec,
                                                                DcTabs dc) {
@@ -286,7 +286,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_pside_weights(const int32_t* pc
     for (int d = threadIdx.x; d < nd; d += ROW_THREADS) {
         int64_t j = off[k];
         for (uint32_t s = r0; s < r1; ++s) {
-            const int32_t x = side[s].x;
+            const int32_t x = side[s].hi.x;
             if (x < 0 || !(x & NBR_PERIODIC)) continue;
             const d4 n = side64[s];
             const double t = exact_t(n, om64 + 3 * d);
