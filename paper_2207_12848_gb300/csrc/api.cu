@@ -169,14 +169,8 @@ void drop_operators(Levels& L) {
     L.dopt.valid = false;
 }
 
-sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
+sweep_status alloc_level_buffers(sweep_ctx* c, Levels& L, int d0, int nd) {
     const int64_t N = c->mesh.N;
-    if (L.nd == nd && L.raw && L.d0 == d0) {
-        L.valid = false;
-        drop_operators(L);
-        return SWEEP_OK;
-    }
-    free_levels(L);
     L.d0 = d0;
     L.nd = nd;
     int bits = dir_bits(nd);
@@ -197,6 +191,18 @@ sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
     return SWEEP_OK;
 }
 
+sweep_status alloc_levels(sweep_ctx* c, Levels& L, int d0, int nd) {
+    if (L.nd == nd && L.raw && L.d0 == d0) {
+        L.valid = false;
+        drop_operators(L);
+        return SWEEP_OK;
+    }
+    free_levels(L);
+    const sweep_status s = alloc_level_buffers(c, L, d0, nd);
+    if (s != SWEEP_OK) free_levels(L);  // all or nothing: a later call must not find some of them
+    return s;
+}
+
 sweep_status run_levelise(sweep_ctx* c, Levels& L, int d0, int nd, long long budget, float* t1, float* t2,
                           int transport = 0) {
     sweep_status s = alloc_levels(c, L, d0, nd);
@@ -204,10 +210,14 @@ sweep_status run_levelise(sweep_ctx* c, Levels& L, int d0, int nd, long long bud
     // scheme (b) tables, [N][nd] each (freed when scheme (a) is levelised again)
     if (transport > 0 && !L.dc_mask) {
         const size_t n = (size_t)c->mesh.N * nd;
-        CK(dev_alloc(&L.dc_mask, sizeof(uint64_t) * n), "alloc scheme (b) tables");
-        CK(dev_alloc(&L.dc_inm, sizeof(uint64_t) * n), "alloc scheme (b) tables");
-        CK(dev_alloc(&L.dc_share32, sizeof(float) * n), "alloc scheme (b) tables");
-        CK(dev_alloc(&L.dc_share64, sizeof(double) * n), "alloc scheme (b) tables");
+        cudaError_t e = dev_alloc(&L.dc_mask, sizeof(uint64_t) * n);
+        if (e == cudaSuccess) e = dev_alloc(&L.dc_inm, sizeof(uint64_t) * n);
+        if (e == cudaSuccess) e = dev_alloc(&L.dc_share32, sizeof(float) * n);
+        if (e == cudaSuccess) e = dev_alloc(&L.dc_share64, sizeof(double) * n);
+        if (e != cudaSuccess) {
+            dfree(L.dc_mask); dfree(L.dc_inm); dfree(L.dc_share32); dfree(L.dc_share64);
+            return cuda_status(c, e, "alloc scheme (b) tables");
+        }
     } else if (transport == 0 && L.dc_mask) {
         dfree(L.dc_mask); dfree(L.dc_inm); dfree(L.dc_share32); dfree(L.dc_share64);
     }
@@ -242,8 +252,9 @@ sweep_status ensure_common(sweep_ctx* c) {
 }
 
 sweep_status ensure_ng(sweep_ctx* c, size_t ng) {
-    if (c->ng_cap >= ng && c->J) return SWEEP_OK;
+    if (c->ng_cap > 0 && c->ng_cap >= ng) return SWEEP_OK;
     dfree(c->J); dfree(c->Jold); dfree(c->Gam); dfree(c->jn); dfree(c->jn1);
+    c->ng_cap = 0;
     size_t n = ng > 0 ? ng : 1;
     CK(dev_alloc(&c->J, sizeof(double) * n), "alloc J");
     CK(dev_alloc(&c->Jold, sizeof(double) * n), "alloc J");
@@ -255,8 +266,9 @@ sweep_status ensure_ng(sweep_ctx* c, size_t ng) {
 }
 
 sweep_status ensure_cm(sweep_ctx* c, size_t n) {
-    if (c->cm_cap >= n && c->cm32) return SWEEP_OK;
+    if (c->cm_cap > 0 && c->cm_cap >= n) return SWEEP_OK;
     dfree(c->cm32); dfree(c->cm64);
+    c->cm_cap = 0;
     size_t m = n > 0 ? n : 1;
     CK(dev_alloc(&c->cm32, sizeof(float2) * m), "alloc sources");
     CK(dev_alloc(&c->cm64, sizeof(double2) * m), "alloc sources");
@@ -732,7 +744,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
         dev_free(d_area); dev_free(d_normal); dev_free(d_fc); dev_free(d_tmp); dev_free(d_flags);
         dev_free(d_off); dev_free(d_bad);
     };
-#define CKM(x, what) do { cudaError_t _e = (x); if (_e != cudaSuccess) { cleanup(); dev_free(d_vol); return cuda_status(c, _e, what); } } while (0)
+#define CKM(x, what) do { cudaError_t _e = (x); if (_e != cudaSuccess) { cleanup(); dev_free(d_vol); free_mesh(c->mesh); return cuda_status(c, _e, what); } } while (0)
     CKM(dev_alloc(&d_vol, sizeof(double) * n_cells), "alloc volume");
     CKM(dev_alloc(&d_area, sizeof(double) * F1), "alloc area");
     CKM(dev_alloc(&d_normal, sizeof(double) * 3 * F1), "alloc normal");
@@ -770,6 +782,7 @@ sweep_status sweep_set_mesh(sweep_ctx* c, int64_t n_cells, const double* volume,
     m.S = S;
     m.NB = NB;
     m.vol = d_vol;
+    d_vol = nullptr;  // the mesh's from here on
     m.mesh_off = off;
     CKM(dev_alloc(&m.rowptr, sizeof(uint32_t) * (n_cells + 1)), "alloc rows");
     CKM(dev_alloc(&m.side, sizeof(SideRec) * ((S > 0 ? S : 1) + 64)), "alloc sides");
@@ -804,6 +817,7 @@ sweep_status sweep_set_directions(sweep_ctx* c, int32_t n_dir, const double* ome
     free_levels(c->lev);
     free_levels(c->adj_lev);
     free_solution(c);
+    c->has_dirs = false;
     std::vector<float4> o32(n_dir), o32lo(n_dir);
     for (int d = 0; d < n_dir; ++d) {
         const double* w = omega + 3 * d;
@@ -1585,6 +1599,7 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     if (c->adj_bytes_I != bI || c->adj_bytes_L != bL) {
         dfree(c->adjI);
         dfree(c->adjL);
+        c->adj_bytes_I = c->adj_bytes_L = 0;
         CK(dev_alloc(&c->adjI, bI > 0 ? bI : 4), "alloc adjoint batch");
         CK(dev_alloc(&c->adjL, bL > 0 ? bL : 4), "alloc adjoint batch");
         c->adj_bytes_I = bI;
