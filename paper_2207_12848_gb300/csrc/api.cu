@@ -1042,7 +1042,7 @@ sweep_status ensure_operator(sweep_ctx* c, Levels& L, const sweep_opts* o, int p
 // BALANCE law (the EXP law reads the mesh rows).
 bool dir_wanted(const sweep_opts* o, int prec, int width, bool transposed) {
     if (!o || o->schedule != SWEEP_SCHED_AUTO || o->geometry_only || o->op_format == SWEEP_OP_LINES || o->lanes_per_task ||
-        o->packets_per_step || o->block_threads || o->blocks_per_sm || o->debug_stall)
+        o->packets_per_step || o->block_threads || o->blocks_per_sm || (o->debug_stall && o->debug_stall < 2))
         return false;
     if (prec == 64 && o->law != SWEEP_LAW_BALANCE) return false;
     return width == 2 || width == 4 || (width == 1 && !transposed);
@@ -1411,7 +1411,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         for (;;) {
             const int parity = !b.sign[cur];
             SweepArgs a = make_args(c, c->lev, prec, cm, b.I[cur], has_pbc ? b.I[prev] : nullptr, G, parity, 0, 0, &o);
-            a.debug_stall = o.debug_stall && n_sweeps == 0;
+            a.debug_stall = n_sweeps > 0 ? 0 : (by_dir ? o.debug_stall : o.debug_stall != 0);
             s = run_sweep(c, c->lev, prec, plain ? SWEEP_SCHED_PLAIN : sched, threads, lanes, bpsm, a, bc32,
                           &t_sweep);
             if (s != SWEEP_OK) return s;

@@ -836,11 +836,17 @@ __global__ void __launch_bounds__(DIR_BOUND)
                     if (++iss < nr) to = is_c ? tab[iss + 1].x : tab[iss + 1].y;
                 }
             };
-            auto need = [&](int lim) {  // rounds below lim have arrived
-                for (; ok && wt < min(lim, nr); ++wt) {
-                    ok = wt < iss && mbar_wait(&bar[ws], ph, a.spin_budget);
-                    ws = ws + 1 == depth ? 0u : ws + 1;
-                    ph ^= ws == 0 ? 1u : 0u;
+            // test only: the wait for this round counts as given up (direction 0; even numbers the rounds of C, odd of E)
+            const int give_up = a.debug_stall >= 2 && d == 0 && (a.debug_stall & 1) == (is_c ? 0 : 1) ? (a.debug_stall - 2) >> 1 : -1;
+            auto passed = [&]() {
+                ++wt;
+                ws = ws + 1 == depth ? 0u : ws + 1;
+                ph ^= ws == 0 ? 1u : 0u;
+            };
+            auto need = [&](int lim) {  // rounds below lim have arrived; after a wait that gave up wt stays at its round
+                while (ok && wt < min(lim, nr)) {
+                    ok = wt < iss && wt != give_up && mbar_wait(&bar[ws], ph, a.spin_budget);
+                    if (ok) passed();
                 }
             };
             if (on) {
@@ -860,12 +866,11 @@ __global__ void __launch_bounds__(DIR_BOUND)
                 __syncwarp();
                 __syncthreads();
             }
-            if (on && *fail <= nr) {  // a bounded wait gave up: report, let the copies in flight land
+            if (on && *fail <= nr) {  // a bounded wait gave up: report, let the copies in flight land (the one waited for first)
                 atomicCAS(a.err, DEV_OK, DEV_TIMEOUT);
-                for (; wt < iss; ++wt) {
+                while (wt < iss) {
                     mbar_wait(&bar[ws], ph, a.spin_budget);
-                    ws = ws + 1 == depth ? 0u : ws + 1;
-                    ph ^= ws == 0 ? 1u : 0u;
+                    passed();
                 }
             }
             __syncwarp();
