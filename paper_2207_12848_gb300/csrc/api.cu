@@ -405,6 +405,13 @@ sweep_status run_sweep(sweep_ctx* c, const Levels& L, int precision, int schedul
     return SWEEP_OK;
 }
 
+// A sweep that gave up has written part of its buffer with the sign of this sweep, which the next sweep of the buffer
+// would take for its own values: start the buffer anew.
+void forget_sweep(sweep_ctx* c, int k) {
+    cudaMemsetAsync(c->sb.I[k], 0, c->sb.bytes, c->st);
+    c->sb.sign[k] = 0;
+}
+
 // ---------------------------------------------------------------------------------------------
 // The periodic iteration (Sec. 2.7) or the source iteration (Alg. 1) as CUDA graphs. The iterations
 // of a solve repeat with a short period: which intensity buffer is swept, the sign parity it is
@@ -581,6 +588,7 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
         st.t_other += to;
         if (hp->err != DEV_OK) {
             c->err = "sweep: a bounded device wait gave up";
+            forget_sweep(c, cur_of(t));
             return SWEEP_ERR_TIMEOUT;
         }
         const int cur = cur_of(t);
@@ -1187,6 +1195,7 @@ sweep_status autotune(sweep_ctx* c, int prec, const void* cm, const float* bc32,
         a.debug_stall = 0;
         sweep_status st = run_sweep(c, c->lev, prec, k.sched, k.threads, k.lanes, k.bpsm, a, bc32, ms);
         if (st == SWEEP_OK) b.sign[tb] = parity;
+        else forget_sweep(c, tb);
         return st;
     };
     // one untimed sweep first (caches, first touch of the buffers), then the best of two per candidate
@@ -1414,7 +1423,10 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
             a.debug_stall = n_sweeps > 0 ? 0 : (by_dir ? o.debug_stall : o.debug_stall != 0);
             s = run_sweep(c, c->lev, prec, plain ? SWEEP_SCHED_PLAIN : sched, threads, lanes, bpsm, a, bc32,
                           &t_sweep);
-            if (s != SWEEP_OK) return s;
+            if (s != SWEEP_OK) {
+                forget_sweep(c, cur);
+                return s;
+            }
             b.sign[cur] = parity;
             ++n_sweeps;
             ++it_scat;
