@@ -177,7 +177,9 @@ __device__ __forceinline__ double block_sum_fixed(double v, double* sh) {
 // cell, into partial[2k], partial[2k+1]. Bound by the FP64 pipe: a direction's flux factor sum A n.Omega over the
 // cell's outflow faces is formed first (three fused multiply-adds a face, none for a face whose FP32 sign says inflow
 // of a vacuum boundary) and meets the G intensities once; n.Omega per face and group took 3.3 ms for the
-// 110,000 boundary cells of 25 meshes, 128 directions, 2 groups.
+// 110,000 boundary cells of 25 meshes, 128 directions, 2 groups. The fused n.Omega may differ in sign from the
+// classification's where it is all rounding; with scheme (a) such a face carries next to nothing, under scheme (b) a
+// chosen face carries its share whatever n.Omega is, so there the mask alone decides.
 template <typename real>
 __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* bcells, const uint32_t* rowptr,
                                                                 const SideRec* side, const d4* side64, const real* I,
@@ -192,6 +194,7 @@ __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* b
     for (int d = threadIdx.x; d < nd; d += ROW_THREADS) {
         const double ox = om64[3 * d], oy = om64[3 * d + 1], oz = om64[3 * d + 2], w = w64[d];
         const float fx = (float)ox, fy = (float)oy, fz = (float)oz;
+        const uint64_t chosen = dc.mask ? dc.mask[(int64_t)c * nd + d] : 0ull;
         double out = 0.0;  // flux factor of the outflow through vacuum faces
         for (uint32_t s = r0; s < r1; ++s) {
             const int4 rec = side[s].hi;
@@ -200,16 +203,15 @@ __global__ void __launch_bounds__(ROW_THREADS) k_boundary_tally(const int32_t* b
                 const float ax = __int_as_float(rec.y), ay = __int_as_float(rec.z), az = __int_as_float(rec.w);
                 if (ax * fx + ay * fy + az * fz < -BAND_REL * (fabsf(ax) + fabsf(ay) + fabsf(az))) continue;
             }
+            // scheme (b): the outflow leaves through a vacuum face only if the cell chose it, with its share
+            if (dc.mask && ((chosen >> (s - r0)) & 1ull)) {
+                out = dadd(out, dc.share64[(int64_t)c * nd + d]);
+                continue;
+            }
             const d4 n = side64[s];
             const double t = fma(n.z, oz, fma(n.y, oy, dmul(n.x, ox)));
             if (t > 0.0) {
-                // scheme (b): the outflow leaves through a vacuum face only if the cell chose it, with its share
-                if (dc.mask) {
-                    const int64_t i = (int64_t)c * nd + d;
-                    if ((dc.mask[i] >> (s - r0)) & 1ull) out = dadd(out, dc.share64[i]);
-                } else {
-                    out = fma(n.w, t, out);
-                }
+                if (!dc.mask) out = fma(n.w, t, out);
             } else if (bc) {
                 const double wa = dmul(w, dmul(n.w, -t));
                 for (int g = 0; g < G; ++g) inj = fma(wa, bc[(size_t)(-1 - rec.x) * G + g], inj);
