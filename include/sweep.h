@@ -97,8 +97,8 @@ typedef struct {
                              nested, the plain schedule or debug_stall, or when capture is refused: host loop) */
     int64_t spin_budget;  /* bound on each device-side wait, in polls (0 = default, about 1 s) */
     int32_t debug_stall;  /* TEST ONLY: 1 makes the first sweep task wait on a word nothing writes; 2 + 2 r (3 + 2 r), where
-                             AUTO sweeps with one block per direction, lets the wait for the r-th copy of direction 0's control
-                             words (entries) count as given up (elsewhere as 1) */
+                             AUTO sweeps two groups under BALANCE with one block per direction, ends the copies of direction
+                             0's control words (entries) before the r-th, whose wait then gives up (elsewhere as 1) */
     int32_t lanes_per_task; /* lanes cooperating on one task in the batched sweep: 1..16, a power of 2 (0 = autotuned);
                                over the assembled operator 2, 4 or 8 (1 runs as 2), and 16 = 8 lanes per task
                                with two tasks per lane group (one group, dataflow schedule; else as 8) */

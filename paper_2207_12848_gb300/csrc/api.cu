@@ -1052,6 +1052,7 @@ bool dir_wanted(const sweep_opts* o, int prec, int width, bool transposed) {
     if (!o || o->schedule != SWEEP_SCHED_AUTO || o->geometry_only || o->op_format == SWEEP_OP_LINES || o->lanes_per_task ||
         o->packets_per_step || o->block_threads || o->blocks_per_sm || (o->debug_stall && o->debug_stall < 2))
         return false;
+    if (o->debug_stall && (o->law != SWEEP_LAW_BALANCE || width != 2 || transposed)) return false;  // the form that tests stop
     if (prec == 64 && o->law != SWEEP_LAW_BALANCE) return false;
     return width == 2 || width == 4 || (width == 1 && !transposed);
 }

@@ -684,7 +684,9 @@ constexpr int DIR_BOUND = 576;
 // 84 directions took 0.92 ms per sweep, with one copying warp for both streams 0.56 ms, as it stands 0.52 ms (the
 // packets of all directions: 0.88 ms). 3000 cells, 16 directions, 2 groups: 0.12 against 0.20 ms; 2^18 cells, 64
 // directions, 2 groups: 1.21 against 1.60 ms.
-template <typename real, int GC, int MODE, int FORM>
+// STOPS (tests only): a form of its own, because the copying warps are part of every level's chain and a condition
+// more in their loop costs 0.5 to 1% of a sweep.
+template <typename real, int GC, int MODE, int FORM, bool STOPS = false>
 __global__ void __launch_bounds__(DIR_BOUND)
     k_sweep_dir(const __grid_constant__ SweepArgs a, const __grid_constant__ DirArgs p) {
     extern __shared__ __align__(128) unsigned char sm[];
@@ -828,25 +830,22 @@ __global__ void __launch_bounds__(DIR_BOUND)
             bool ok = true;
             // offsets of round iss and of the next one (read an iteration before they are used)
             uint32_t at = is_c ? tab[0].x : tab[0].y, to = is_c ? tab[1].x : tab[1].y;
+            // STOPS: the copies of one stream of direction 0 end at a round, whose wait then gives up at once
+            int stop = nr;
+            if (STOPS && d == 0 && (a.debug_stall & 1) == (is_c ? 0 : 1)) stop = min(nr, (a.debug_stall - 2) >> 1);
             auto issue = [&](int lim) {  // rounds below lim
-                if (iss < min(lim, nr)) {
+                if (iss < min(lim, stop)) {
                     bulk_load(ring + is * slot_bytes, src + (size_t)at * unit, (to - at) * unit, &bar[is], pol);
                     at = to;
                     is = is + 1 == depth ? 0u : is + 1;
                     if (++iss < nr) to = is_c ? tab[iss + 1].x : tab[iss + 1].y;
                 }
             };
-            // test only: the wait for this round counts as given up (direction 0; even numbers the rounds of C, odd of E)
-            const int give_up = a.debug_stall >= 2 && d == 0 && (a.debug_stall & 1) == (is_c ? 0 : 1) ? (a.debug_stall - 2) >> 1 : -1;
-            auto passed = [&]() {
-                ++wt;
-                ws = ws + 1 == depth ? 0u : ws + 1;
-                ph ^= ws == 0 ? 1u : 0u;
-            };
-            auto need = [&](int lim) {  // rounds below lim have arrived; after a wait that gave up wt stays at its round
-                while (ok && wt < min(lim, nr)) {
-                    ok = wt < iss && wt != give_up && mbar_wait(&bar[ws], ph, a.spin_budget);
-                    if (ok) passed();
+            auto need = [&](int lim) {  // rounds below lim have arrived
+                for (; ok && wt < min(lim, nr); ++wt) {
+                    ok = wt < iss && mbar_wait(&bar[ws], ph, a.spin_budget);
+                    ws = ws + 1 == depth ? 0u : ws + 1;
+                    ph ^= ws == 0 ? 1u : 0u;
                 }
             };
             if (on) {
@@ -868,9 +867,15 @@ __global__ void __launch_bounds__(DIR_BOUND)
             }
             if (on && *fail <= nr) {  // a bounded wait gave up: report, let the copies in flight land (the one waited for first)
                 atomicCAS(a.err, DEV_OK, DEV_TIMEOUT);
-                while (wt < iss) {
+                if (!ok) {  // back to the round whose wait gave up
+                    ph ^= ws == 0 ? 1u : 0u;
+                    ws = ws == 0 ? depth - 1 : ws - 1;
+                    --wt;
+                }
+                for (; wt < iss; ++wt) {
                     mbar_wait(&bar[ws], ph, a.spin_budget);
-                    passed();
+                    ws = ws + 1 == depth ? 0u : ws + 1;
+                    ph ^= ws == 0 ? 1u : 0u;
                 }
             }
             __syncwarp();
@@ -901,7 +906,12 @@ const void* dir_kernel(int GC, int mode) {
     }
 }
 template <typename real>
-const void* dir_kernel(int GC, int mode, int form) {
+const void* dir_kernel(int GC, int mode, int form, bool stops) {
+    if (stops) {
+        if constexpr (sizeof(real) == 4)
+            if (form == MID) return (const void*)k_sweep_dir<real, 2, PK_BALANCE, MID, true>;
+        return (const void*)k_sweep_dir<real, 2, PK_BALANCE, NARROW, true>;
+    }
     if constexpr (sizeof(real) == 4)
         if (form == MID) return dir_kernel<real, MID>(GC, mode);
     return dir_kernel<real, NARROW>(GC, mode);
@@ -1089,7 +1099,8 @@ cudaError_t launch_sweep_dir(const SweepArgs& a, const DirOp& P, int mode, int s
     DirArgs p;
     p.E = P.E; p.C = P.C; p.meta = P.meta; p.rtab = P.rtab; p.rstride = P.rstride; p.R = P.R; p.Fs = P.Fs; p.W = P.W;
     p.off_cm = P.off_cm; p.off_c = P.off_c; p.off_e = P.off_e; p.c_slot = P.c_slot; p.e_slot = P.e_slot;
-    const void* f = P.real_bytes == 8 ? dir_kernel<double>(P.GC, mode, P.form) : dir_kernel<float>(P.GC, mode, P.form);
+    const void* f = P.real_bytes == 8 ? dir_kernel<double>(P.GC, mode, P.form, a.debug_stall >= 2)
+                                      : dir_kernel<float>(P.GC, mode, P.form, a.debug_stall >= 2);
     cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};

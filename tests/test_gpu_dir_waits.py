@@ -1,6 +1,6 @@
 """The sweep by direction when a wait for its operator copies gives up: status TIMEOUT, and the next solve on the same
-context is right. The give-up is reported by the kernel itself (debug_stall >= 2); the copies in flight still land, and
-every wait stays bounded."""
+context is right. The copies of one stream stop at a round (debug_stall >= 2), so that the wait for it gives up at once; the copies in
+flight still land, and every wait stays bounded."""
 import numpy as np
 import pytest
 
@@ -32,7 +32,7 @@ def test_copy_wait_gives_up(ctx, copy, stream, n_dir):
 
 
 def test_copy_past_the_last_is_waited_for(ctx):
-    p = configs.voronoi_small(600, n_dir=4, seed=32)
+    p = configs.voronoi_small(600, n_dir=4, n_groups=2, seed=32)
     ctx.set_mesh(p.mesh)
     ctx.set_directions(p.omega, p.weight)
     ctx.set_material(p.kappa_abs, p.emissivity)
