@@ -66,10 +66,12 @@ __device__ __forceinline__ double weighted_sum(const real* I, size_t stride, int
 }
 
 // Largest of a non-negative value over the block, into *dmax by one atomic per block (one per value serialises in L2:
-// 0.50 ms for 10^6 values). A NaN (the change between two infinite values) counts as none. Blocks of 256 threads.
+// 0.50 ms for 10^6 values). A NaN (the change between two infinite values) counts as none; it is told by its bits, the FP64
+// pipe being the bound. Blocks of 256 threads.
 __device__ __forceinline__ void block_max(double v, unsigned long long* dmax) {
     __shared__ unsigned long long s_max[8];
-    unsigned long long x = v > 0.0 ? (unsigned long long)__double_as_longlong(v) : 0ull;
+    unsigned long long x = (unsigned long long)__double_as_longlong(v);
+    if (x > 0x7ff0000000000000ull) x = 0ull;
     for (int o = 16; o > 0; o >>= 1) {
         const unsigned long long y = __shfl_xor_sync(0xffffffffu, x, o);
         x = y > x ? y : x;
