@@ -1101,7 +1101,9 @@ cudaError_t launch_sweep_dir(const SweepArgs& a, const DirOp& P, int mode, int s
     p.off_cm = P.off_cm; p.off_c = P.off_c; p.off_e = P.off_e; p.c_slot = P.c_slot; p.e_slot = P.e_slot;
     const void* f = P.real_bytes == 8 ? dir_kernel<double>(P.GC, mode, P.form, a.debug_stall >= 2)
                                       : dir_kernel<float>(P.GC, mode, P.form, a.debug_stall >= 2);
-    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)P.smem);
+    // the most that any plan takes, not this plan's: the attribute belongs to the kernel, and a context of another
+    // thread may set it between here and the launch
+    cudaError_t e = cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_BLOCK);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)std::min(a.nd, sms));
