@@ -93,7 +93,8 @@ struct DirBuild {
     uint2* rtab;               // [nd][RC + 1] {C offset / 16, E offset / 256} of each round
     int2* tot;                 // [nd] slices, rounds
     DirMeta* meta;             // [nd]
-    int32_t* stat;             // [0] does not apply, [1] most far sources of a slice, [2] most C bytes, [3] most E bytes
+    int32_t* stat;             // [0] does not apply, [1] most far sources of a slice, [2] bound on a round's E bytes
+    uint32_t e_slot, quad_b;   // E bytes of a round's slot, bytes of a quad
     unsigned char *E, *C;
     const uint32_t* rowptr;
     const SideRec* side;
@@ -127,6 +128,15 @@ __device__ uint64_t entry_mask(const DirBuild& a, uint32_t c, int d, float* P) {
     }
     return m;
 }
+
+// The plan's slots turned out too small for the E of a round: the host plans again with the bound, and until then
+// nothing more is counted (a second count of 2^18 cells, 128 directions costs 2.1 ms of a 15 ms solve).
+// Raises *p to v, by an atomic only where it would change it: of the hundreds of thousands of blocks and slices few do, and
+// atomics on one address come one after the other.
+__device__ __forceinline__ void raise_stat(int32_t* p, int v) {
+    if (v > *(volatile int32_t*)p) atomicMax(p, v);
+}
+__device__ __forceinline__ bool slot_too_small(const DirBuild& a) { return (uint32_t)a.stat[2] > a.e_slot; }
 
 __device__ __forceinline__ int level_slices(int n) { return (n + 31) >> 5; }
 // A level of n slices has ceil(n / W) rounds of equal size, so its last round is not a small remainder.
@@ -176,6 +186,7 @@ __global__ void __launch_bounds__(1024) k_dir_slices(DirBuild a) {
 
 // First round of every level.
 __global__ void __launch_bounds__(1024) k_dir_rounds(DirBuild a) {
+    if (slot_too_small(a)) return;
     const int d = blockIdx.x;
     const int32_t* nr = a.nround + (size_t)d * a.lcap;
     const int n = level_scan(a.depth[d], a.transposed, [&](int L) { return nr[L]; }, a.rbase + (size_t)d * a.lcap);
@@ -204,7 +215,7 @@ __device__ int cut_rounds(const uint32_t* sfar, int ns, int per, uint32_t Fs, F 
 template <bool WRITE>
 __global__ void __launch_bounds__(128) k_dir_cut(DirBuild a) {
     const int L = blockIdx.x * 128 + threadIdx.x, d = blockIdx.y;
-    if (L >= a.depth[d]) return;
+    if (L >= a.depth[d] || slot_too_small(a)) return;
     const int ns = level_slices(a.dcnt[(size_t)d * a.cap + L]), s0 = a.sbase[(size_t)d * a.lcap + L];
     if (s0 + ns > a.SC) return;
     const uint32_t* sf = a.sfar + (size_t)d * a.SC + s0;
@@ -222,10 +233,10 @@ __global__ void __launch_bounds__(128) k_dir_cut(DirBuild a) {
 }
 
 // One block per (level, direction): the tasks sorted by their quads (counting sort, longest first) and put
-// into slices.
+// into slices. A round's slices follow one another, so none has more quads than a level's first round.
 constexpr int PLACE_THREADS = 128;
 __global__ void __launch_bounds__(PLACE_THREADS) k_dir_place(DirBuild a) {
-    __shared__ int s_bin[MAX_Q + 1], s_end[MAX_Q + 1];
+    __shared__ int s_bin[MAX_Q + 1], s_end[MAX_Q + 1], s_first;
     const int L = blockIdx.x, d = blockIdx.y;
     if (L >= a.depth[d]) return;
     const int n = a.dcnt[(size_t)d * a.cap + L];
@@ -234,6 +245,7 @@ __global__ void __launch_bounds__(PLACE_THREADS) k_dir_place(DirBuild a) {
     if (s0 + ns > a.SC) return;
     const size_t o = ((size_t)d * a.SC + s0) * 32;
     if (threadIdx.x <= MAX_Q) s_bin[threadIdx.x] = 0;
+    if (threadIdx.x == 0) s_first = 0;
     __syncthreads();
     for (int i = threadIdx.x; i < n; i += PLACE_THREADS) {
         float P;
@@ -271,7 +283,10 @@ __global__ void __launch_bounds__(PLACE_THREADS) k_dir_place(DirBuild a) {
         int q = MAX_Q;
         while (q > 1 && s_end[q] <= i * 32) --q;
         a.nq[(size_t)d * a.SC + s0 + i] = (uint32_t)q;
+        if (i < round_slices(ns, a.W)) atomicAdd(&s_first, q);
     }
+    __syncthreads();
+    if (threadIdx.x == 0) raise_stat(&a.stat[2], s_first * (int)a.quad_b);
 }
 
 // ring slot of an entry's source, or ~0 where the value has to be staged. level_end: the place after the
@@ -285,7 +300,7 @@ __device__ __forceinline__ uint32_t near_slot(const DirBuild& a, int d, int32_t 
 // Far entries of each slice (one block per level of a direction, a warp per slice).
 __global__ void __launch_bounds__(128) k_dir_count(DirBuild a) {
     const int L = blockIdx.x, d = blockIdx.y;
-    if (L >= a.depth[d]) return;
+    if (L >= a.depth[d] || slot_too_small(a)) return;
     const int ns = level_slices(a.dcnt[(size_t)d * a.cap + L]), s0 = a.sbase[(size_t)d * a.lcap + L];
     if (s0 + ns > a.SC) return;
     const uint32_t end = (uint32_t)(s0 + ns) * 32u;
@@ -306,7 +321,7 @@ __global__ void __launch_bounds__(128) k_dir_count(DirBuild a) {
         if (lane == 0) {
             a.sfar[(size_t)d * a.SC + s0 + k] = (uint32_t)far;
             a.lend[(size_t)d * a.SC + s0 + k] = end;
-            atomicMax(&a.stat[1], far);
+            raise_stat(&a.stat[1], far);
         }
     }
 }
@@ -345,7 +360,7 @@ template <typename real>
 __global__ void __launch_bounds__(1024) k_dir_offsets(DirBuild a) {
     const int d = blockIdx.x;
     const int2 t = a.tot[d];
-    if (t.x > a.SC || t.y > a.RC) return;
+    if (t.x > a.SC || t.y > a.RC || slot_too_small(a)) return;
     const uint32_t* nq = a.nq + (size_t)d * a.SC;
     uint32_t* eoff = a.eoff + (size_t)d * (a.SC + 1);
     uint32_t* coff = a.coff + (size_t)d * (a.RC + 1);
@@ -354,15 +369,8 @@ __global__ void __launch_bounds__(1024) k_dir_offsets(DirBuild a) {
     const uint32_t e = block_scan(t.x, [&](int i) { return nq[i] * (quad_bytes<real>() / 256u); }, eoff);
     const uint32_t c = block_scan(t.y, [&](int i) { return c_bytes<real>(ri[i].y, nf[i]) / 16u; }, coff);
     __syncthreads();
-    int ce = 0, cc = 0;
-    for (int i = threadIdx.x; i <= t.y; i += 1024) {
+    for (int i = threadIdx.x; i <= t.y; i += 1024)
         a.rtab[(size_t)d * (a.RC + 1) + i] = make_uint2(coff[i], i < t.y ? eoff[ri[i].x] : e);
-        if (i == t.y) break;
-        ce = max(ce, (int)(eoff[ri[i].x + ri[i].y] - eoff[ri[i].x]) * 256);
-        cc = max(cc, (int)c_bytes<real>(ri[i].y, nf[i]));
-    }
-    atomicMax(&a.stat[2], cc);
-    atomicMax(&a.stat[3], ce);
     if (threadIdx.x == 0) {
         if (e >= (1u << 24) || c >= (1u << 28)) atomicOr(&a.stat[0], 1);  // offsets are kept in 32 bits
         a.meta[d].e_bytes = (int64_t)e * 256;
@@ -436,12 +444,18 @@ __global__ void __launch_bounds__(128) k_dir_write(DirBuild a) {
         rec.cell = c;
         rec.P = (real)a.P[t];
         if (sizeof(real) == 8 && c != PAD_CELL) {
+            // P_c in FP64, in row order. The FP64 pipe bounds this build, so the sides that the classification calls
+            // inflow are left out.
             double P = 0.0;
-            for (uint32_t s = r0; s < a.rowptr[c + 1]; ++s) {
+            const auto add = [&](uint32_t s) {
                 const d4 nn = a.side64[s];
                 const double tt = exact_t(nn, a.om64 + 3 * d);
                 if (tt > 0.0) P = __dadd_rn(P, __dmul_rn(nn.w, tt));
-            }
+            };
+            const uint32_t r1 = a.rowptr[c + 1], n = r1 - r0;
+            uint32_t m = ~(uint32_t)a.info[(int64_t)c * a.nd + d].z & (n >= 32u ? ~0u : (1u << n) - 1u);
+            for (; m; m &= m - 1) add(r0 + (uint32_t)(__ffs((int)m) - 1));
+            for (uint32_t s = r0 + 32; s < r1; ++s) add(s);
             rec.P = (real)P;
         }
         tasks[k * 32u + lane] = rec;
@@ -966,7 +980,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     P.Fs = std::max(256, 128 + 64 * P.W);
     const uint32_t cb = real_bytes == 8 ? c_bytes<double>((uint32_t)P.W, (uint32_t)P.Fs) : c_bytes<float>((uint32_t)P.W, (uint32_t)P.Fs);
     P.c_slot = (cb + 127u) & ~127u;
-    // E of a round: a guess at its longest slices' quads, corrected below
+    // E of a round: a guess at its longest slices' quads, corrected below by the bound that placing the tasks gives
     P.e_slot = (uint32_t)((P.W == 1 ? 6.0 : (P.W == 2 ? 5.0 : (P.W <= 4 ? 4.0 : 3.4))) * P.W) * (uint32_t)(32 * (4 * real_bytes + 8));
     if (!layout(P)) return cudaSuccess;
     DirBuild a;
@@ -1033,16 +1047,17 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     const bool dc = L.transport > 0 && !transposed;
     a.dc_inm = dc ? L.dc_inm : nullptr; a.dc_share32 = dc ? L.dc_share32 : nullptr; a.dc_share64 = dc ? L.dc_share64 : nullptr;
     a.R = P.R; a.A = P.A; a.Fs = P.Fs;
+    a.quad_b = (uint32_t)(32 * (4 * real_bytes + 8));
     if ((e = cudaMemsetAsync(a.stat, 0, 16, st))) return e;
     const dim3 lev((unsigned)nl, (unsigned)nd), levt((unsigned)((nl + 127) / 128), (unsigned)nd);
     P.launches = 0;
     for (int attempt = 0; attempt < 5; ++attempt) {
-        a.R = P.R; a.A = P.A; a.Fs = P.Fs;
+        a.R = P.R; a.A = P.A; a.Fs = P.Fs; a.e_slot = P.e_slot;
         if (attempt == 0) {
             k_dir_slices<<<nd, 1024, 0, st>>>(a);
             k_dir_place<<<lev, PLACE_THREADS, 0, st>>>(a);
         }
-        if ((e = cudaMemsetAsync(a.stat + 1, 0, 12, st))) return e;
+        if ((e = cudaMemsetAsync(a.stat + 1, 0, 4, st))) return e;
         k_dir_count<<<lev, 128, 0, st>>>(a);
         k_dir_cut<false><<<levt, 128, 0, st>>>(a);
         k_dir_rounds<<<nd, 1024, 0, st>>>(a);
@@ -1051,7 +1066,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         else k_dir_offsets<float><<<nd, 1024, 0, st>>>(a);
         k_dir_bases<<<1, 1024, 0, st>>>(P.meta, nd, total, (uint32_t*)(ws + o_sc));
         P.launches += attempt == 0 ? 8 : 6;
-        int32_t stat[4] = {};
+        int32_t stat[3] = {};
         int64_t tt[2] = {};
         if ((e = cudaMemcpyAsync(stat, a.stat, sizeof stat, cudaMemcpyDeviceToHost, st))) return e;
         if ((e = cudaMemcpyAsync(tt, total, sizeof tt, cudaMemcpyDeviceToHost, st))) return e;
@@ -1059,7 +1074,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         P.e_bytes = tt[0];
         P.c_bytes = tt[1];
         if (stat[0]) return cudaSuccess;
-        // a slice's far sources, and a round's C and E, must fit their slots
+        // a round's E, and a slice's far sources, must fit their slots
         bool fits = true;
         if (stat[1] > P.Fs) {
             P.Fs = (stat[1] + 31) & ~31;
@@ -1067,8 +1082,8 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
             P.c_slot = (cbn + 127u) & ~127u;
             fits = false;
         }
-        if ((uint32_t)stat[3] > P.e_slot) {
-            P.e_slot = ((uint32_t)stat[3] + 127u) & ~127u;
+        if ((uint32_t)stat[2] > P.e_slot) {
+            P.e_slot = ((uint32_t)stat[2] + 127u) & ~127u;
             fits = false;
         }
         if (fits) {
