@@ -165,8 +165,7 @@ int dir_bits(int nd) {
 void drop_operators(Levels& L) {
     L.op_valid = false;
     L.pkt.valid = false;
-    L.dop.valid = false;
-    L.dopt.valid = false;
+    for (DirOp* P : {&L.dop, &L.dopt}) P->known = P->valid = false;
 }
 
 sweep_status alloc_level_buffers(sweep_ctx* c, Levels& L, int d0, int nd) {
@@ -1057,12 +1056,16 @@ bool dir_wanted(const sweep_opts* o, int prec, int width, bool transposed) {
     return width == 2 || width == 4 || (width == 1 && !transposed);
 }
 
-// The per-direction operator of the cached levels for values of `width` numbers, built once per levelisation
-// and width. P.valid stays false where it does not apply or does not fit in device memory.
+// The per-direction operator of the cached levels for values of `width` numbers, planned and built once per levelisation
+// and width. P.valid stays false where it does not apply (remembered: a plan costs up to a count of all entries and
+// a synchronisation) or does not fit in device memory (tried again when there is room).
 sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int prec, int width, float* t_ms) {
     const int rb = prec == 64 ? 8 : 4;
-    if (P.valid && P.real_bytes == rb && P.GC == width) return SWEEP_OK;
-    P.valid = false;
+    if (P.known && P.real_bytes == rb && P.GC == width && (P.valid || !P.room || !op_fits(P.room))) return SWEEP_OK;
+    P.known = P.valid = false;
+    P.real_bytes = rb;
+    P.GC = width;
+    P.room = 0;
     ScopedEvent e0, e1;
     cudaEventRecord(e0, c->st);
     bool ok = false;
@@ -1075,6 +1078,7 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int 
         if (!op_fits((size_t)n) || dev_alloc(&p, (size_t)n) != cudaSuccess) {
             cudaGetLastError();
             p = nullptr;
+            P.room = (size_t)n;
             return false;
         }
         cap = n;
@@ -1085,6 +1089,7 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int 
         CK(dir_write(P, c->st), "write operator");
         P.valid = true;
     }
+    P.known = true;
     c->launches += P.launches;
     cudaEventRecord(e1, c->st);
     CK(cudaEventSynchronize(e1), "assemble operator");

@@ -454,6 +454,8 @@ struct DirOp {
     uint32_t e_slot = 0, c_slot = 0, off_cm = 0, off_c = 0, off_e = 0, smem = 0;
     int launches = 0;                  // kernels of the last build
     std::vector<char> args;            // build arguments kept between plan and write
+    bool known = false;                // planned for the current levels: valid says whether it applies
+    size_t room = 0;                   // where only device memory was lacking: the bytes it asked for
     bool valid = false;                // written for the current levels
 };
 

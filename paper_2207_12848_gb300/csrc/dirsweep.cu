@@ -960,6 +960,7 @@ bool layout(DirOp& P) {
 cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int real_bytes, int GC, const double* om64_all,
                      const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok) {
     *ok = false;
+    P.launches = 0;
     const int nd = L.nd, nl = L.n_levels;
     if (nl < 1 || m.max_row > 64 || m.NB >= (1ll << 30) || !L.by_dir) return cudaSuccess;
     double dsum = 0;
@@ -972,8 +973,6 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     // 5.6 ms. FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. With more
     // than two directions per SM the directions that wait cost more than the levels gain.
     if (width > (real_bytes == 8 ? 512.0 : 256.0) || nd > 2 * sms) return cudaSuccess;
-    P.real_bytes = real_bytes;
-    P.GC = GC;
     // one round per level where the workers suffice (FP64 sums are bound by the FP64 pipe: four warps fill it)
     P.W = std::min(real_bytes == 8 ? Form<NARROW>::W : Form<MID>::W, std::max(1, (int)(1.2 * (width / 32.0 + 0.5) + 0.5)));
     P.form = P.W <= Form<NARROW>::W ? NARROW : MID;
@@ -1012,11 +1011,14 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         if (L.dir_ws) dev_free(L.dir_ws);
         L.dir_ws = nullptr;
         L.dir_ws_bytes = 0;
+        // no room: the packets take their place
+        P.room = off;
         if (off + ((size_t)2 << 30) > dev_available()) return cudaSuccess;
-        if (dev_alloc(&L.dir_ws, off) != cudaSuccess) {  // no room: the packets take their place
+        if (dev_alloc(&L.dir_ws, off) != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;
         }
+        P.room = 0;
         L.dir_ws_bytes = off;
     }
     const size_t keep = ((sizeof(DirMeta) * nd + 255) & ~(size_t)255) + 8 * nR;
@@ -1026,6 +1028,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         P.meta_bytes = 0;
         if (dev_alloc(&P.meta, keep) != cudaSuccess) {
             cudaGetLastError();
+            P.room = keep;
             return cudaSuccess;
         }
         P.meta_bytes = keep;
@@ -1050,7 +1053,6 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     a.quad_b = (uint32_t)(32 * (4 * real_bytes + 8));
     if ((e = cudaMemsetAsync(a.stat, 0, 16, st))) return e;
     const dim3 lev((unsigned)nl, (unsigned)nd), levt((unsigned)((nl + 127) / 128), (unsigned)nd);
-    P.launches = 0;
     for (int attempt = 0; attempt < 5; ++attempt) {
         a.R = P.R; a.A = P.A; a.Fs = P.Fs; a.e_slot = P.e_slot;
         if (attempt == 0) {
