@@ -76,6 +76,7 @@ struct sweep_ctx {
     // autotuner: schedule and block size per (precision, G)
     int tuned[2][9][3][4] = {};  // [precision][groups][operator form OPF_*] -> schedule, threads, lanes, blocks/SM
     int64_t launches = 0;  // kernels launched by this context
+    long long dir_clock = 0;  // requests for per-direction operators so far
     PeriodicTable ptab;          // periodic-inflow weights, rebuilt at the start of each periodic solve
     MemPool pool;                // device memory given up by the buffers above and kept for the next ones
     cudaStream_t gst = nullptr;  // capture/replay stream of the iteration graphs
@@ -117,6 +118,28 @@ void dfree(T*& p) {
     p = nullptr;
 }
 
+void free_dir(DirOp& P) {
+    dfree(P.E); dfree(P.C); dfree(P.meta);
+    P = DirOp();
+}
+
+// the per-direction operators that the present call does not sweep over, and the tables of their builds (MemPool::set_spare)
+bool spare_dirs(void* ctx) {
+    Levels& L = static_cast<sweep_ctx*>(ctx)->lev;
+    bool any = false;
+    for (DirOp& P : L.dirs) {
+        if ((!P.E && !P.C) || &P == L.dop || &P == L.dopt) continue;
+        free_dir(P);
+        any = true;
+    }
+    if (L.dir_ws && !L.dir_building) {
+        dfree(L.dir_ws);
+        L.dir_ws_bytes = 0;
+        any = true;
+    }
+    return any;
+}
+
 void free_levels(Levels& L) {
     dfree(L.raw); dfree(L.task); dfree(L.trec); dfree(L.info); dfree(L.level); dfree(L.word); dfree(L.lvl_cnt); dfree(L.pad_off);
     dfree(L.lev_chunk); dfree(L.seg_off); dfree(L.op); dfree(L.dlev);
@@ -124,9 +147,7 @@ void free_levels(Levels& L) {
         dfree(P->pk); dfree(P->meta); dfree(P->lev_pk); dfree(P->grp); dfree(P->lev_grp); dfree(P->cnt);
         dfree(P->off); dfree(P->scan); dfree(P->flag);
     }
-    for (DirOp* P : {&L.dop, &L.dopt}) {
-        dfree(P->E); dfree(P->C); dfree(P->meta);
-    }
+    for (DirOp& P : L.dirs) free_dir(P);
     dfree(L.dir_ws);
     dfree(L.lfill);
     dfree(L.dc_mask); dfree(L.dc_inm); dfree(L.dc_share32); dfree(L.dc_share64);
@@ -165,7 +186,8 @@ int dir_bits(int nd) {
 void drop_operators(Levels& L) {
     L.op_valid = false;
     L.pkt.valid = false;
-    for (DirOp* P : {&L.dop, &L.dopt}) P->known = P->valid = false;
+    for (DirOp& P : L.dirs) P.known = P.valid = false;
+    L.dop = L.dopt = nullptr;
 }
 
 sweep_status alloc_level_buffers(sweep_ctx* c, Levels& L, int d0, int nd) {
@@ -379,7 +401,7 @@ sweep_status run_sweep(sweep_ctx* c, const Levels& L, int precision, int schedul
         }
     } else if (schedule == SCHED_DIR) {
         c->last_kernel = SWEEP_KERNEL_PACKED;
-        CKL(launch_sweep_dir(a, a.reverse ? L.dopt : L.dop, pk_mode(a), c->sms, c->st), "sweep launch");
+        CKL(launch_sweep_dir(a, a.reverse ? *L.dopt : *L.dop, pk_mode(a), c->sms, c->st), "sweep launch");
     } else {
         const int fmt = a.pk ? OPF_PACKETS : (a.op ? OPF_LINES : OPF_NONE);
         // without an assembled operator the adjoint, the EXP law and scheme (b) run in the generic kernel
@@ -531,7 +553,7 @@ sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void*
         a.lanes = lanes;
         if (sched == SCHED_DIR) {
             kid = SWEEP_KERNEL_PACKED;
-            e = launch_sweep_dir(a, c->lev.dop, pk_mode(a), c->sms, gs);
+            e = launch_sweep_dir(a, *c->lev.dop, pk_mode(a), c->sms, gs);
         } else {
             e = launch_sweep(a, prec, c->sms * per_sm, threads, gs, &kid);
         }
@@ -671,6 +693,7 @@ sweep_status sweep_create(sweep_ctx** out, int device, void* stream) {
     c->device = device;
     c->st = (cudaStream_t)stream;
     PoolScope pool_scope(&c->pool);
+    c->pool.set_spare(spare_dirs, c);
     cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, device);
     int coop = 0;
     cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, device);
@@ -935,8 +958,9 @@ int wanted_format(sweep_ctx* c, const Levels& L, const sweep_opts* o, int prec) 
 }
 
 // device memory for an operator of `bytes`, keeping a margin for the solve buffers allocated later
+constexpr size_t OP_MARGIN = (size_t)2 << 30;
 bool op_fits(size_t bytes) {
-    return bytes + (size_t)(2ull << 30) <= dev_available();
+    return dev_room(bytes + OP_MARGIN);
 }
 
 // Plans and writes a packed operator of the levels L (transposed: the adjoint's), growing its buffers
@@ -1056,16 +1080,41 @@ bool dir_wanted(const sweep_opts* o, int prec, int width, bool transposed) {
     return width == 2 || width == 4 || (width == 1 && !transposed);
 }
 
-// The per-direction operator of the cached levels for values of `width` numbers, planned and built once per levelisation
-// and width. P.valid stays false where it does not apply (remembered: a plan costs up to a count of all entries and
-// a synchronisation) or does not fit in device memory (tried again when there is room).
-sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int prec, int width, float* t_ms) {
+// The place of the operator for these values: its own, or that of the one not asked for for longest.
+DirOp& dir_place(Levels& L, bool transposed, int real_bytes, int width) {
+    DirOp* old = &L.dirs[0];
+    for (DirOp& P : L.dirs) {
+        if (P.used && P.transposed == transposed && P.real_bytes == real_bytes && P.GC == width) return P;
+        if (P.used < old->used) old = &P;
+    }
+    return *old;
+}
+
+// Points L.dop (transposed: L.dopt) to the per-direction operator of the cached levels for values of `width` numbers, planned
+// and built once per levelisation and kind; null where it does not apply (remembered: a plan costs up to a count of all
+// entries and a synchronisation) or does not fit in device memory (tried again when there is room).
+sweep_status ensure_dir(sweep_ctx* c, Levels& L, bool transposed, int prec, int width, float* t_ms) {
     const int rb = prec == 64 ? 8 : 4;
-    if (P.known && P.real_bytes == rb && P.GC == width && (P.valid || !P.room || !op_fits(P.room))) return SWEEP_OK;
-    P.known = P.valid = false;
+    const DirOp*& found = transposed ? L.dopt : L.dop;
+    found = nullptr;
+    DirOp& P = dir_place(L, transposed, rb, width);
+    const bool same = P.known && P.transposed == transposed && P.real_bytes == rb && P.GC == width;
+    P.transposed = transposed;
     P.real_bytes = rb;
     P.GC = width;
+    P.used = ++c->dir_clock;
+    found = &P;  // keeps its buffers from being given up
+    if (same && (P.valid || !P.room || !dev_room(P.room + OP_MARGIN, false))) {
+        if (!P.valid) found = nullptr;
+        return SWEEP_OK;
+    }
+    P.known = P.valid = false;
     P.room = 0;
+    struct Building {
+        bool& b;
+        explicit Building(bool& x) : b(x) { b = true; }
+        ~Building() { b = false; }
+    } building(L.dir_building);
     ScopedEvent e0, e1;
     cudaEventRecord(e0, c->st);
     bool ok = false;
@@ -1090,6 +1139,7 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, DirOp& P, bool transposed, int 
         P.valid = true;
     }
     P.known = true;
+    if (!P.valid) found = nullptr;
     c->launches += P.launches;
     cudaEventRecord(e1, c->st);
     CK(cudaEventSynchronize(e1), "assemble operator");
@@ -1282,11 +1332,12 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     float tc = 0, tl = 0, top = 0;
     sweep_status s = ensure_levels(c, &o, &tc, &tl);
     if (s != SWEEP_OK) return s;
+    c->lev.dop = c->lev.dopt = nullptr;
     bool by_dir = !plain && dir_wanted(&o, prec, c->G, false);
     if (by_dir) {
-        s = ensure_dir(c, c->lev, c->lev.dop, false, prec, c->G, &top);
+        s = ensure_dir(c, c->lev, false, prec, c->G, &top);
         if (s != SWEEP_OK) return s;
-        by_dir = c->lev.dop.valid;
+        by_dir = c->lev.dop != nullptr;
     }
     if (!by_dir) {
         s = ensure_merged(c, c->lev);
@@ -1331,7 +1382,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     int bpsm = o.blocks_per_sm;
     if (by_dir) {
         sched = SCHED_DIR;
-        threads = 64 * c->lev.dop.W + 64;
+        threads = 64 * c->lev.dop->W + 64;
         lanes = bpsm = 1;
     }
     // the EXP law: no tuning, the dataflow schedule (packets: two per warp step)
@@ -1660,13 +1711,14 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
         if (nb == D) {
             L = &c->lev;
             s = ensure_levels(c, &o, &a1, &a2);
+            L->dop = L->dopt = nullptr;
             if (s == SWEEP_OK && !plain && !coupled && dir_wanted(&o, prec, G, false)) {
-                s = ensure_dir(c, *L, L->dop, false, prec, G, &tasm);
-                fwd_dir = L->dop.valid;
+                s = ensure_dir(c, *L, false, prec, G, &tasm);
+                fwd_dir = L->dop != nullptr;
             }
             if (s == SWEEP_OK && !plain && dir_wanted(&o, prec, 2 * G, true)) {
-                s = ensure_dir(c, *L, L->dopt, true, prec, 2 * G, &tasm);
-                tr_dir = L->dopt.valid;
+                s = ensure_dir(c, *L, true, prec, 2 * G, &tasm);
+                tr_dir = L->dopt != nullptr;
             }
             if (s == SWEEP_OK && !(tr_dir && (fwd_dir || coupled))) s = ensure_merged(c, *L);
             if (s == SWEEP_OK && !fwd_dir && !coupled) s = ensure_operator(c, *L, &o, prec, &tasm);

@@ -346,7 +346,8 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, long l
 // up are kept, LIMIT bytes of them at most, and handed out again for a request that fills four fifths of one or more.
 // Everything a context does is ordered on its stream, so a block may be handed out while work on its former contents
 // is queued. Blocks that nothing asked for during KEEP solves or adjoints are freed, as are all of them when an
-// allocation fails and when the context is destroyed. Measured on a step that sets a mesh and a material (67,581
+// allocation fails and when the context is destroyed. An allocation that still fails asks the context for what it can
+// do without (set_spare) before it gives up. Measured on a step that sets a mesh and a material (67,581
 // cells, 48 directions) and solves: 6.9 ms -> 4.35 ms; a solve and adjoint of 2^18 cells 6.6 -> 5.75 ms.
 class MemPool {
 public:
@@ -358,6 +359,9 @@ public:
     void end_of_call();             // a solve or adjoint has ended: free what has not been asked for lately
     void trim(int keep);            // free the blocks given up more than `keep` calls ago (0: all)
     size_t cached() const { return cached_; }
+    // spare(arg) gives up memory that the context can build again, and returns whether there was any
+    void set_spare(bool (*spare)(void*), void* arg) { spare_ = spare; spare_arg_ = arg; }
+    bool spare() { return spare_ && spare_(spare_arg_); }
 
 private:
     struct Block {
@@ -368,6 +372,8 @@ private:
     std::vector<Block> live_, free_;
     size_t cached_ = 0;
     int epoch_ = 0;
+    bool (*spare_)(void*) = nullptr;
+    void* spare_arg_ = nullptr;
 };
 // the pool of the context whose entry point this thread is in
 class PoolScope {
@@ -384,7 +390,8 @@ cudaError_t dev_alloc_bytes(void** p, size_t bytes);
 void dev_free(void* p);
 template <typename T>
 cudaError_t dev_alloc(T** p, size_t bytes) { return dev_alloc_bytes(reinterpret_cast<void**>(p), bytes); }
-size_t dev_available();  // bytes an allocation could get: free on the device, and kept by the pool
+// whether an allocation could get so much: free on the device, kept by the pool, or (give_up) spare
+bool dev_room(size_t bytes, bool give_up = true);
 
 // One face side of a cell's row: the neighbour code with the outward area vector in FP32, and the area vector minus its
 // FP32 value. The two halves share a 32-byte sector: packing reads both of every inflow side and nothing of
@@ -448,7 +455,9 @@ struct DirOp {
     size_t meta_bytes = 0;             // of meta and rtab (one allocation)
     uint2* rtab = nullptr;             // [nd][rstride] offsets of every round
     int rstride = 0;
+    bool transposed = false;
     int real_bytes = 0, GC = 0;        // values it was planned for
+    long long used = 0;                // when it was last asked for (0: never)
     int W = 0, R = 0, A = 0, Fs = 0;   // slices per round, ring places, rounds fetched ahead, far sources per stage
     int form = 0;                      // of the kernel: narrow or wider levels
     uint32_t e_slot = 0, c_slot = 0, off_cm = 0, off_c = 0, off_e = 0, smem = 0;
@@ -463,7 +472,13 @@ struct Levels {
     bool valid = false;
     bool by_dir = false;         // levelised one direction per block: per-direction level lists are there
     bool merged = false;         // the level-major task list of all directions is there
-    DirOp dop, dopt;             // per-direction operator, forward and transposed
+    // Per-direction operators, one for each direction of transport, precision and number of values that was asked for
+    // lately: calls that take turns (FP32 and FP64, a solve and its adjoint) find theirs again. Rebuilding one for
+    // 2^18 cells, 64 directions, 2 groups costs 4.5 ms (FP64 11.9) beside a sweep of 1.2 (8.5).
+    static constexpr int DIR_OPS = 4;
+    DirOp dirs[DIR_OPS];
+    const DirOp *dop = nullptr, *dopt = nullptr;  // those of the present call, forward and transposed
+    bool dir_building = false;   // the tables below are in use
     void* dir_ws = nullptr;      // tables their builds work in
     size_t dir_ws_bytes = 0;
     int d0 = 0, nd = 0;

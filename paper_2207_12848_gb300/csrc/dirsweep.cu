@@ -1013,7 +1013,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         L.dir_ws_bytes = 0;
         // no room: the packets take their place
         P.room = off;
-        if (off + ((size_t)2 << 30) > dev_available()) return cudaSuccess;
+        if (!dev_room(off + ((size_t)2 << 30))) return cudaSuccess;
         if (dev_alloc(&L.dir_ws, off) != cudaSuccess) {
             cudaGetLastError();
             return cudaSuccess;

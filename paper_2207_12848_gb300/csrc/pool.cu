@@ -34,6 +34,11 @@ cudaError_t MemPool::alloc(void** p, size_t bytes) {
         trim(0);
         e = cudaMalloc(p, n);
     }
+    if (e == cudaErrorMemoryAllocation && spare()) {
+        cudaGetLastError();
+        trim(0);
+        e = cudaMalloc(p, n);
+    }
     if (e != cudaSuccess) {
         *p = nullptr;
         return e;
@@ -84,10 +89,13 @@ void dev_free(void* p) {
     if (t_pool) t_pool->free(p);
     else cudaFree(p);
 }
-size_t dev_available() {
-    size_t free_b = 0, total_b = 0;
-    cudaMemGetInfo(&free_b, &total_b);
-    return free_b + (t_pool ? t_pool->cached() : 0);
+bool dev_room(size_t bytes, bool give_up) {
+    const auto fits = [&] {
+        size_t free_b = 0, total_b = 0;
+        cudaMemGetInfo(&free_b, &total_b);
+        return bytes <= free_b + (t_pool ? t_pool->cached() : 0);
+    };
+    return fits() || (give_up && t_pool && t_pool->spare() && fits());
 }
 
 }  // namespace sw

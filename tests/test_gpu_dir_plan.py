@@ -1,7 +1,9 @@
 """The operator of the sweep by direction: planned once per levelisation, kept per precision and number of groups."""
 import numpy as np
 import pytest
+import torch
 
+from paper_2207_12848_gb300 import Context
 from synth import configs
 from synth.fields import fibonacci_directions
 from synth.mesh import Mesh, column_mesh, lattice_mesh
@@ -37,3 +39,81 @@ def test_plan_that_does_not_apply_is_made_once(ctx, precision):
     assert st[0]["t_assemble_ms"] == st[1]["t_assemble_ms"] == 0.0
     # what a solve of kept levels launches besides: AUTO's preparation of the source before it looks up its schedule
     assert st[0]["kernel_launches"] == st[1]["kernel_launches"] <= ref["kernel_launches"] + 1
+
+
+def load(ctx, p):
+    ctx.set_mesh(p.mesh)
+    ctx.set_directions(p.omega, p.weight)
+    ctx.set_material(p.kappa_abs, p.emissivity)
+
+
+def test_calls_of_two_precisions_take_turns(gpu_lib):
+    # a solve and an adjoint in FP32 and in FP64 on one context: each finds its operator again, and answers as on a context of its own
+    p = configs.voronoi_small(6000, n_dir=12, n_groups=2, seed=51)
+    g = np.random.default_rng(3).normal(size=p.kappa_abs.shape)
+    want = {}
+    for precision in (32, 64):
+        with Context(0) as c:
+            load(c, p)
+            want[precision] = c.solve(precision=precision)[0], c.adjoint(dl_dJ=g, precision=precision)[:2]
+    with Context(0) as c:
+        load(c, p)
+        for turn in range(3):
+            for precision in (32, 64):
+                J, _, st, _ = c.solve(precision=precision)
+                gk, ge, sa = c.adjoint(dl_dJ=g, precision=precision)
+                assert st["lanes_used"] == 1 and sa["schedule_used"] == 1
+                assert (st["t_assemble_ms"] == 0.0) == (sa["t_assemble_ms"] == 0.0) == (turn > 0)
+                assert np.array_equal(J, want[precision][0])
+                assert np.array_equal(gk, want[precision][1][0]) and np.array_equal(ge, want[precision][1][1])
+
+
+def test_more_kinds_than_are_kept(gpu_lib):
+    # six kinds (three numbers of groups, two precisions) in turn: the one not asked for for longest makes room
+    p = configs.voronoi_small(3000, n_dir=7, n_groups=4, seed=52, periodic_box=True)
+    kinds = [(G, precision) for G in (1, 2, 4) for precision in (32, 64)]
+    it = dict(tol_pbc=0.0, max_it_pbc=2)
+
+    def solve(c, G, precision):
+        c.set_material(p.kappa_abs[:, :G].copy(), p.emissivity[:, :G].copy())
+        return c.solve(precision=precision, **it)
+
+    want = {}
+    for k in kinds:
+        with Context(0) as c:
+            load(c, p)
+            want[k] = solve(c, *k)[0]
+    with Context(0) as c:
+        load(c, p)
+        for k in kinds + kinds[::-1] + kinds:
+            J, _, st, _ = solve(c, *k)
+            assert st["lanes_used"] == 1 and np.array_equal(J, want[k])
+        c.set_directions(-p.omega, p.weight)  # other levels: none of the kept ones holds any more
+        for k in kinds:
+            J, _, st, _ = solve(c, *k)
+            assert st["t_assemble_ms"] > 0.0 and not np.array_equal(J, want[k])
+        c.set_directions(p.omega, p.weight)
+        for k in kinds:
+            assert np.array_equal(solve(c, *k)[0], want[k])
+
+
+def test_kept_operators_make_room(gpu_lib):
+    # operators of other calls are given up before a call runs out of memory
+    p = configs.voronoi_small(60000, n_dir=48, seed=53)
+    kw = dict(precision=64, law="exp", schedule="dataflow")  # reads the mesh rows: about 100 MB more
+    with Context(0) as c:
+        load(c, p)
+        want = c.solve(**kw)[0]
+    with Context(0) as c:
+        load(c, p)
+        first = [c.solve(precision=q)[0] for q in (32, 64)]
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info(0)[0]
+        held = torch.empty(free - (8 << 20), dtype=torch.uint8, device="cuda")
+        try:
+            assert np.array_equal(c.solve(**kw)[0], want)
+        finally:
+            del held
+            torch.cuda.empty_cache()
+        for q, J in zip((32, 64), first):
+            assert np.array_equal(c.solve(precision=q)[0], J)
