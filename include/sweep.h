@@ -62,8 +62,8 @@ enum {
 };
 
 /* AUTO, with lanes_per_task, packets_per_step, block_threads and blocks_per_sm left at 0, op_format not LINES and
- * geometry_only 0, sweeps narrow levels (up to 256 tasks per direction and level on average, in FP64 512) with one
- * block per direction: barriers between the levels of that direction only, and the operator in a stream of its
+ * geometry_only 0, sweeps narrow levels (up to 256 tasks per direction and level on average, in FP64 512, or 96
+ * with values of 4) with one block per direction: barriers between the levels of that direction only, and the operator in a stream of its
  * own order. Values of 1, 2 or 4 groups (transposed: 2 or 4 split groups), rows of up to 64 face sides, in FP64 the
  * BALANCE law. sweep_stats then reports schedule_used LEVEL, kernel_used PACKED, lanes_used and
  * blocks_per_sm_used 1. */

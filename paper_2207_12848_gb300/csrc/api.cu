@@ -1110,6 +1110,7 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, bool transposed, int prec, int 
     }
     P.known = P.valid = false;
     P.room = 0;
+    P.launches = 0;
     struct Building {
         bool& b;
         explicit Building(bool& x) : b(x) { b = true; }

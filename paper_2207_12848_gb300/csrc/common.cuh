@@ -589,7 +589,7 @@ cudaError_t pack_write(const DevMesh& m, const Levels& L, PackedOp& P, bool tran
 // the level-major task list of levels made by direction (what every sweep but the per-direction one reads)
 cudaError_t merge_levels(const DevMesh& m, Levels& L, cudaStream_t st);
 cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int real_bytes, int GC, const double* om64_all,
-                     const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok);
+                     const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok, int w_max = 1 << 30);
 cudaError_t dir_write(DirOp& P, cudaStream_t st);
 cudaError_t launch_sweep_dir(const SweepArgs& a, const DirOp& P, int mode, int sms, cudaStream_t st);
 cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const float4* om32_all,

@@ -958,9 +958,8 @@ bool layout(DirOp& P) {
 // Plans the operator of the levels L for values of GC numbers of real_bytes: places, slices, rounds, offsets.
 // *ok = false where this form does not apply; P.e_bytes and P.c_bytes are what the streams need.
 cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int real_bytes, int GC, const double* om64_all,
-                     const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok) {
+                     const float4* om32_all, const float4* om32lo_all, int sms, cudaStream_t st, bool* ok, int w_max) {
     *ok = false;
-    P.launches = 0;
     const int nd = L.nd, nl = L.n_levels;
     if (nl < 1 || m.max_row > 64 || m.NB >= (1ll << 30) || !L.by_dir) return cudaSuccess;
     double dsum = 0;
@@ -970,18 +969,26 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     // round takes. FP32: 204 tasks per level (2^18 cells, 64 directions) 1.21 against 1.60 ms for the packets of
     // all directions, 196 (scheme (b), 60 directions) 0.08 against 0.11 ms; 584 (2^21 cells, 128 directions) 9.7
     // against 10.6 ms, which the longer build does not earn back; 957 (25 meshes, 2 groups) 7.1 against
-    // 5.6 ms. FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. With more
-    // than two directions per SM the directions that wait cost more than the levels gain.
-    if (width > (real_bytes == 8 ? 512.0 : 256.0) || nd > 2 * sms) return cudaSuccess;
+    // 5.6 ms. FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. Four FP64 values
+    // leave room for three workers and a short ring: 92 tasks per level 10.4 against 12.3 ms (67,581 cells, 32 directions),
+    // 160 already 25.1 against 19.5. With more than two directions per SM the directions that wait cost more than the
+    // levels gain.
+    const double line = real_bytes == 4 ? 256.0 : (GC == 4 ? 96.0 : 512.0);
+    if (width > line || nd > 2 * sms) return cudaSuccess;
     // one round per level where the workers suffice (FP64 sums are bound by the FP64 pipe: four warps fill it)
     P.W = std::min(real_bytes == 8 ? Form<NARROW>::W : Form<MID>::W, std::max(1, (int)(1.2 * (width / 32.0 + 0.5) + 0.5)));
+    P.W = std::min(P.W, w_max);
+    const auto narrower = [&]() -> cudaError_t {  // the regions of a round leave no ring (FP64, four values): fewer workers
+        if (P.W <= 1) return cudaSuccess;
+        return dir_plan(m, L, P, transposed, real_bytes, GC, om64_all, om32_all, om32lo_all, sms, st, ok, P.W - 1);
+    };
     P.form = P.W <= Form<NARROW>::W ? NARROW : MID;
     P.Fs = std::max(256, 128 + 64 * P.W);
     const uint32_t cb = real_bytes == 8 ? c_bytes<double>((uint32_t)P.W, (uint32_t)P.Fs) : c_bytes<float>((uint32_t)P.W, (uint32_t)P.Fs);
     P.c_slot = (cb + 127u) & ~127u;
     // E of a round: a guess at its longest slices' quads, corrected below by the bound that placing the tasks gives
     P.e_slot = (uint32_t)((P.W == 1 ? 6.0 : (P.W == 2 ? 5.0 : (P.W <= 4 ? 4.0 : 3.4))) * P.W) * (uint32_t)(32 * (4 * real_bytes + 8));
-    if (!layout(P)) return cudaSuccess;
+    if (!layout(P)) return narrower();
     DirBuild a;
     a.cap = L.dlev_cap;
     a.dcnt = L.dlev;
@@ -1094,7 +1101,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
             memcpy(P.args.data(), &a, sizeof a);
             return cudaGetLastError();
         }
-        if (!layout(P)) return cudaSuccess;
+        if (!layout(P)) return narrower();
     }
     return cudaSuccess;
 }
