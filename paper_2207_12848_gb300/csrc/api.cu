@@ -202,7 +202,6 @@ sweep_status alloc_level_buffers(sweep_ctx* c, Levels& L, int d0, int nd) {
     CK(dev_alloc(&L.raw, sizeof(uint32_t) * L.task_cap), "alloc task list");
     CK(dev_alloc(&L.info, sizeof(int4) * N * nd), "alloc classification");
     CK(dev_alloc(&L.level, sizeof(int32_t) * N * nd), "alloc levels");
-    CK(dev_alloc(&L.word, sizeof(unsigned long long) * N * nd), "alloc levels");
     CK(dev_alloc(&L.lvl_cnt, sizeof(int32_t) * (N + 2)), "alloc level counts");
     CK(dev_alloc(&L.pad_off, sizeof(uint32_t) * (N + 2)), "alloc level offsets");
     CK(dev_alloc(&L.lev_chunk, sizeof(int64_t) * (N + 2)), "alloc level chunks");
@@ -228,6 +227,7 @@ sweep_status run_levelise(sweep_ctx* c, Levels& L, int d0, int nd, long long bud
                           int transport = 0) {
     sweep_status s = alloc_levels(c, L, d0, nd);
     if (s != SWEEP_OK) return s;
+    if (!L.trec && !L.word) CK(dev_alloc(&L.word, sizeof(unsigned long long) * (size_t)c->mesh.N * nd), "alloc levels");
     // scheme (b) tables, [N][nd] each (freed when scheme (a) is levelised again)
     if (transport > 0 && !L.dc_mask) {
         const size_t n = (size_t)c->mesh.N * nd;

@@ -505,7 +505,10 @@ struct Levels {
     float* dc_share32 = nullptr;
     double* dc_share64 = nullptr;
     int32_t* level = nullptr;    // [nd][N]
-    unsigned long long* word = nullptr;  // [nd][N] levelisation: {sides that release, upwind cells still unsolved}
+    // [nd][N] levelisation: {sides that release, upwind cells still unsolved}. Dead once the levels are made, so it
+    // stands in the task records' memory where these exist, and gives way to them (8 bytes a task, 4.3 GB at 2^22 cells, 128 directions).
+    unsigned long long* word = nullptr;
+    unsigned long long* words() const { return word ? word : reinterpret_cast<unsigned long long*>(trec); }
     int32_t* lvl_cnt = nullptr;  // [N+2]
     uint32_t* pad_off = nullptr; // [N+2] start of each level in the padded list
     int64_t* lev_chunk = nullptr;  // device [n_levels+1] chunk (32-task) offsets

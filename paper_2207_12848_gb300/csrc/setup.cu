@@ -1438,7 +1438,7 @@ cudaError_t classify(const DevMesh& m, Levels& L, const float4* om32, const floa
     if (tot > 0)
         k_classify<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, om32, om32lo, om64,
                                                L.info, L.level, L.raw, L.lvl_cnt, L.cshift,
-                                               per_direction ? L.raw : nullptr, n0, L.word);
+                                               per_direction ? L.raw : nullptr, n0, L.words());
     return cudaGetLastError();
 }
 
@@ -1459,7 +1459,11 @@ cudaError_t ensure_seg(Levels& L, int nlev) {
 cudaError_t alloc_merged(Levels& L) {
     cudaError_t e = cudaSuccess;
     if (!L.task) e = dev_alloc(&L.task, sizeof(uint32_t) * L.task_cap);
-    if (e == cudaSuccess && !L.trec) e = dev_alloc(&L.trec, sizeof(int4) * L.task_cap);
+    if (e == cudaSuccess && !L.trec) {
+        dev_free(L.word);
+        L.word = nullptr;
+        e = dev_alloc(&L.trec, sizeof(int4) * L.task_cap);
+    }
     return e;
 }
 
@@ -1487,7 +1491,7 @@ cudaError_t levelise_by_direction(const DevMesh& m, Levels& L, const float4* om3
     int32_t* ovf = depth + nd;
     DirLevArgs a;
     a.N = m.N; a.nd = nd; a.cap = cap; a.long_rows = m.max_row > 32; a.rowptr = m.rowptr; a.ids = m.ids;
-    a.side = m.side; a.side64 = m.side64; a.om32 = om32; a.om64 = om64; a.word = L.word; a.level = L.level;
+    a.side = m.side; a.side64 = m.side64; a.om32 = om32; a.om64 = om64; a.word = L.words(); a.level = L.level;
     a.dlist = L.raw; a.n0 = n0; a.dcnt = dcnt; a.dbase = dbase;
     a.dc_mask = L.transport > 0 ? L.dc_mask : nullptr;
     a.depth = depth; a.overflow = ovf;
@@ -1623,7 +1627,7 @@ cudaError_t levelise(const DevMesh& m, Levels& L, const double* om64_all, const 
             k_dc_choose<<<nblk(tot), 256, 0, st>>>(N, nd, L.transport, m.rowptr, m.side64, om64, L.dc_mask,
                                                    L.dc_share32, L.dc_share64, bad);
             k_dc_count<<<nblk(tot), 256, 0, st>>>(N, nd, m.rowptr, m.side, m.side64, om32, om64, m.twin, L.dc_mask,
-                                                  L.dc_inm, L.level, L.raw, n0, L.word);
+                                                  L.dc_inm, L.level, L.raw, n0, L.words());
         }
         int hbad = 0;
         if ((e = cudaMemcpyAsync(&hbad, bad, sizeof(int), cudaMemcpyDeviceToHost, st))) return e;

@@ -148,3 +148,28 @@ def test_fp64_four_values(gpu_lib, n, kind, by_dir):
         assert a[-1]["schedule_used"] == (1 if by_dir else 2) and b[-1]["schedule_used"] == 2
         for x, y in zip(a[:2], b[:2]):
             assert np.max(np.abs(x - y)) <= 1e-12 * np.max(np.abs(y))
+
+
+def test_levels_hold_no_more_than_their_arrays(gpu_lib):
+    # 64^3 cells, 64 directions: per task the lists, records, classification and levels (44 bytes) and the intensities (4);
+    # the levelisation's words (8) stand in the records' memory once these are made
+    m = lattice_mesh(64)
+    om, w = fibonacci_directions(64, seed=6)
+    tasks = m.n_cells * 64
+    torch.cuda.synchronize()
+    torch.cuda.empty_cache()
+    with Context(0) as c:
+        c.set_mesh(m)
+        c.set_directions(om, w)
+        c.set_material(np.full((m.n_cells, 1), 0.5), np.ones((m.n_cells, 1)))
+        kw = dict(schedule="dataflow", geometry_only=1, lanes_per_task=4)
+        before = torch.cuda.mem_get_info(0)[0]
+        J = c.solve(**kw)[0]
+        for _ in range(6):  # blocks that nothing asked for are given back
+            c.solve(**kw)
+        used = before - torch.cuda.mem_get_info(0)[0]
+        # besides: 32 padding tasks for each possible level in the list (24 bytes each), tables of levels, per-cell arrays
+        extra = 32 * m.n_cells * 24 + 3 * 4 * 64 * 65536 + 100 * m.n_cells
+        assert used <= 48 * tasks + extra + (16 << 20)
+        assert np.array_equal(c.solve(relevel=1, **kw)[0], J)
+        assert before - torch.cuda.mem_get_info(0)[0] <= used
