@@ -1333,26 +1333,11 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     float tc = 0, tl = 0, top = 0;
     sweep_status s = ensure_levels(c, &o, &tc, &tl);
     if (s != SWEEP_OK) return s;
-    c->lev.dop = c->lev.dopt = nullptr;
-    bool by_dir = !plain && dir_wanted(&o, prec, c->G, false);
-    if (by_dir) {
-        s = ensure_dir(c, c->lev, false, prec, c->G, &top);
-        if (s != SWEEP_OK) return s;
-        by_dir = c->lev.dop != nullptr;
-    }
-    if (!by_dir) {
-        s = ensure_merged(c, c->lev);
-        if (s != SWEEP_OK) return s;
-        s = ensure_operator(c, c->lev, &o, prec, &top);
-        if (s != SWEEP_OK) return s;
-    }
-    S.t_ms[0] = tc;
-    S.t_ms[1] = tl;
-    S.t_ms[5] = top;
     const int64_t N = c->mesh.N;
     const int G = c->G, D = c->D;
     const size_t NG = (size_t)N * G;
     const bool has_pbc = c->mesh.n_pcells > 0;
+    // the solve's own buffers before the operators, which make do with the memory that is left
     s = ensure_ng(c, NG);
     if (s != SWEEP_OK) return s;
     s = ensure_cm(c, NG);
@@ -1376,6 +1361,22 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         if (s != SWEEP_OK) return s;
         bc32 = c->bc32;
     }
+    c->lev.dop = c->lev.dopt = nullptr;
+    bool by_dir = !plain && dir_wanted(&o, prec, c->G, false);
+    if (by_dir) {
+        s = ensure_dir(c, c->lev, false, prec, c->G, &top);
+        if (s != SWEEP_OK) return s;
+        by_dir = c->lev.dop != nullptr;
+    }
+    if (!by_dir) {
+        s = ensure_merged(c, c->lev);
+        if (s != SWEEP_OK) return s;
+        s = ensure_operator(c, c->lev, &o, prec, &top);
+        if (s != SWEEP_OK) return s;
+    }
+    S.t_ms[0] = tc;
+    S.t_ms[1] = tl;
+    S.t_ms[5] = top;
     SolveBuf& b = c->sb;
     const void* cm = prec == 64 ? (const void*)c->cm64 : (const void*)c->cm32;
     int sched = o.schedule, threads = o.block_threads ? o.block_threads : 256;
