@@ -142,7 +142,7 @@ typedef struct {
     double res_pbc_mean;
     double emitted, injected, absorbed, escaped; /* photons/s over all cells and groups (FP64) */
     double defect;             /* (emitted + injected - absorbed - escaped) / (emitted + injected) */
-    double t_ms[8];            /* 0 classify, 1 levelise, 2 sweeps, 3 tallies+updates, 4 total, 5 operator
+    double t_ms[8];            /* 0 classify, 1 levelise (with the merged task list, when this call makes it), 2 sweeps, 3 tallies+updates, 4 total, 5 operator
                                   assembly, 6 (adjoint) the transposed sweeps within 2 (CUDA events) */
     double updates;            /* cell x direction x group updates done by all sweeps */
     double updates_per_s;      /* updates / (t_ms[4] / 1000) */

@@ -1150,10 +1150,18 @@ sweep_status ensure_dir(sweep_ctx* c, Levels& L, bool transposed, int prec, int 
     return SWEEP_OK;
 }
 
-// the level-major task list of the cached levels
-sweep_status ensure_merged(sweep_ctx* c, Levels& L) {
-    if (!L.merged) c->launches += 4;
+// the level-major task list of the cached levels (part of the levelisation, made when a sweep first needs it)
+sweep_status ensure_merged(sweep_ctx* c, Levels& L, float* t_ms) {
+    if (L.merged) return SWEEP_OK;
+    ScopedEvent e0, e1;
+    cudaEventRecord(e0, c->st);
+    c->launches += 4;
     CK(merge_levels(c->mesh, L, c->st), "merge levels");
+    cudaEventRecord(e1, c->st);
+    CK(cudaEventSynchronize(e1), "merge levels");
+    float ms = 0;
+    cudaEventElapsedTime(&ms, e0, e1);
+    *t_ms += ms;
     return SWEEP_OK;
 }
 
@@ -1369,7 +1377,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         by_dir = c->lev.dop != nullptr;
     }
     if (!by_dir) {
-        s = ensure_merged(c, c->lev);
+        s = ensure_merged(c, c->lev, &tl);
         if (s != SWEEP_OK) return s;
         s = ensure_operator(c, c->lev, &o, prec, &top);
         if (s != SWEEP_OK) return s;
@@ -1722,13 +1730,13 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
                 s = ensure_dir(c, *L, true, prec, 2 * G, &tasm);
                 tr_dir = L->dopt != nullptr;
             }
-            if (s == SWEEP_OK && !(tr_dir && (fwd_dir || coupled))) s = ensure_merged(c, *L);
+            if (s == SWEEP_OK && !(tr_dir && (fwd_dir || coupled))) s = ensure_merged(c, *L, &a2);
             if (s == SWEEP_OK && !fwd_dir && !coupled) s = ensure_operator(c, *L, &o, prec, &tasm);
             if (s == SWEEP_OK && !tr_dir) s = ensure_transposed(c, *L, &o, prec, &tasm);
         } else {
             s = run_levelise(c, c->adj_lev, d0, nb, budget_of(&o), &a1, &a2);
             L = &c->adj_lev;
-            if (s == SWEEP_OK) s = ensure_merged(c, *L);
+            if (s == SWEEP_OK) s = ensure_merged(c, *L, &a2);
         }
         if (s != SWEEP_OK) return s;
         tcl += a1;

@@ -173,3 +173,19 @@ def test_levels_hold_no_more_than_their_arrays(gpu_lib):
         assert used <= 48 * tasks + extra + (16 << 20)
         assert np.array_equal(c.solve(relevel=1, **kw)[0], J)
         assert before - torch.cuda.mem_get_info(0)[0] <= used
+
+
+def test_merge_counts_as_levelisation(gpu_lib):
+    # the task list of all directions, made when a sweep first needs it, is in the levelisation's time
+    p = configs.voronoi_small(20000, n_dir=16, seed=55)
+    with Context(0) as c:
+        load(c, p)
+        assert c.solve()[2]["lanes_used"] == 1  # by direction: no such list
+        st = c.solve(schedule="dataflow")[2]
+        assert 0.0 < st["t_levelise_ms"] < st["t_total_ms"]
+        assert c.solve(schedule="dataflow")[2]["t_levelise_ms"] == 0.0
+        c.set_material(p.kappa_abs, p.emissivity)
+        c.set_directions(p.omega, p.weight)
+        c.solve()
+        st = c.adjoint(dl_dJ=np.ones((20000, 1)), schedule="dataflow")[2]
+        assert st["t_levelise_ms"] > 0.0
