@@ -28,6 +28,9 @@
  *     arrays are [n_cells][n_groups].
  *   - One context drives one GPU and one CUDA stream. Calls on one context must
  *     not overlap (the context is not thread-safe).
+ *   - A context keeps up to 1 GiB of device memory that its buffers gave up, for its next ones: until four solves or
+ *     adjoints have not asked for it, an allocation of any context of the process fails, or it is destroyed. Other
+ *     users of the GPU see that memory as taken.
  */
 #ifndef SWEEP_H
 #define SWEEP_H

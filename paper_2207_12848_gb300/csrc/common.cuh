@@ -5,6 +5,7 @@
 #include <stdint.h>
 
 #include <cstddef>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -347,28 +348,33 @@ __device__ __forceinline__ bool grid_sync(GridBar* bar, unsigned nblocks, long l
 // Everything a context does is ordered on its stream, so a block may be handed out while work on its former contents
 // is queued. Blocks that nothing asked for during KEEP solves or adjoints are freed, as are all of them when an
 // allocation fails and when the context is destroyed. An allocation that still fails asks the context for what it can
-// do without (set_spare) before it gives up. Measured on a step that sets a mesh and a material (67,581
+// do without (set_spare), and every other context of the process for its kept blocks, before it gives up. Measured on a step that sets a mesh and a material (67,581
 // cells, 48 directions) and solves: 6.9 ms -> 4.35 ms; a solve and adjoint of 2^18 cells 6.6 -> 5.75 ms.
 class MemPool {
 public:
     static constexpr int KEEP = 4;
     static constexpr size_t LIMIT = (size_t)1 << 30;
+    MemPool();
     ~MemPool();
+    MemPool(const MemPool&) = delete;
+    MemPool& operator=(const MemPool&) = delete;
     cudaError_t alloc(void** p, size_t bytes);
     void free(void* p);
     void end_of_call();             // a solve or adjoint has ended: free what has not been asked for lately
     void trim(int keep);            // free the blocks given up more than `keep` calls ago (0: all)
-    size_t cached() const { return cached_; }
+    size_t cached();
     // spare(arg) gives up memory that the context can build again, and returns whether there was any
     void set_spare(bool (*spare)(void*), void* arg) { spare_ = spare; spare_arg_ = arg; }
     bool spare() { return spare_ && spare_(spare_arg_); }
 
 private:
+    cudaError_t allocate(void** p, size_t bytes);  // from the device, giving up kept blocks until it succeeds
     struct Block {
         void* p;
         size_t bytes;
         int epoch;
     };
+    std::mutex m_;  // a context is used by one thread at a time, but its kept blocks may be asked back by another
     std::vector<Block> live_, free_;
     size_t cached_ = 0;
     int epoch_ = 0;
