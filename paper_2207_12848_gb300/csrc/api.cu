@@ -358,6 +358,7 @@ SweepArgs make_args(sweep_ctx* c, const Levels& L, int precision, const void* cm
     a.nd = L.nd;
     a.rowptr = c->mesh.rowptr;
     a.side = c->mesh.side;
+    a.ids = c->mesh.ids;
     a.side64 = c->mesh.side64;
     a.om32 = c->om32 + L.d0;
     a.om32lo = c->om32lo + L.d0;

@@ -553,6 +553,7 @@ struct SweepArgs {
     int nd;               // directions of this batch
     const uint32_t* rowptr;
     const SideRec* side;
+    const int32_t* ids;   // [N][32] neighbour codes of the first 32 sides
     const d4* side64;
     const float4* om32;   // [nd]
     const float4* om32lo; // [nd] low parts of the directions

@@ -1340,7 +1340,8 @@ __device__ __forceinline__ void plain_task(const SweepArgs& a, uint32_t entry) {
         if (g < G) acc[g] = a.law ? 0.0 : (a.reverse ? __dmul_rn(a.w64[dl], cm[g].x) : cm[g].x);
     double P = 0.0;
     for (uint32_t s = r0; s < r1; ++s) {
-        const int32_t nb = a.side[s].hi.x;
+        // the code alone, 4 bytes a side: the 32-byte record is for kernels that need the area vector too
+        const int32_t nb = s - r0 < 32u ? a.ids[(size_t)c * 32 + (s - r0)] : a.side[s].hi.x;
         const d4 n = a.side64[s];
         const double t = exact_t(n, om64);
         if (t == 0.0) continue;
