@@ -508,7 +508,7 @@ struct LoopState {
 // periodic iteration). *done = false (nothing run) when the graphs cannot be captured; the caller then
 // runs the host loop from the same state.
 sweep_status graph_loop(sweep_ctx* c, const sweep_opts& o, int prec, const void* cm, const float* bc32, int sched,
-                        int threads, int lanes, int bpsm, int nblk, LoopState& st, bool* done) {
+                        int threads, int lanes, int bpsm, LoopState& st, bool* done) {
     *done = false;
     const bool pbc = c->mesh.n_pcells > 0;
     const bool scat = c->has_scat;
@@ -1459,7 +1459,7 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
         ls.prev = prev;
         ls.conv_pbc = conv_pbc;
         ls.conv_scat = conv_scat;
-        s = graph_loop(c, o, prec, cm, bc32, sched, threads, lanes, bpsm, nblk, ls, &graphed);
+        s = graph_loop(c, o, prec, cm, bc32, sched, threads, lanes, bpsm, ls, &graphed);
         if (s != SWEEP_OK) return s;
         if (graphed) {
             cur = ls.cur;
@@ -1549,11 +1549,11 @@ sweep_status solve_impl(sweep_ctx* c, const sweep_opts* opts_in, double* J_out, 
     b.last = fin;
     // final tallies: absorbed/emitted from the last tally, escaped/injected over boundary cells
     CKL(launch_tally(prec, o.law ? c->Imean : b.I[fin], N, G, D, 0, c->w64, c->wsum, c->mesh.vol, c->ka, c->em, c->J,
-                    c->Gam, c->partial, nblk, c->st), "tally");
+                    c->Gam, c->partial, c->st), "tally");
     CKL(launch_reduce_sum(c->partial, nblocks256(NG), c->red, c->st), "reduce");
     if (c->mesh.n_bcells > 0) {
         const DcTabs dct = dc_tabs(c, c->lev);
-        CKL(launch_boundary_tally(prec, c->mesh, b.I[fin], G, D, 0, c->om64, c->w64, c->bc, c->partial, nblk, c->st,
+        CKL(launch_boundary_tally(prec, c->mesh, b.I[fin], G, D, 0, c->om64, c->w64, c->bc, c->partial, c->st,
                                   &dct),
            "boundary tally");
         CKL(launch_reduce_sum(c->partial, (int)c->mesh.n_bcells, c->red + 2, c->st), "reduce");

@@ -620,7 +620,7 @@ cudaError_t launch_prep_adjoint_src(int64_t N, int G, const double* vol, const d
                                     cudaStream_t st);
 cudaError_t launch_tally(int precision, const void* I, int64_t N, int G, int nd, int d0, const double* w64,
                          double wsum, const double* vol, const double* ka, const double* em, double* J,
-                         double* Gam, double* partial, int nblk, cudaStream_t st);
+                         double* Gam, double* partial, cudaStream_t st);
 // scheme (b) tables of a solve ([N][nd] chosen outflow sides and FP64 shares, per side the twin's row
 // position); a null pointer to it, or a null mask, means scheme (a)
 struct DcTabs {
@@ -630,7 +630,7 @@ struct DcTabs {
 };
 cudaError_t launch_boundary_tally(int precision, const DevMesh& m, const void* I, int G, int nd, int d0,
                                   const double* om64, const double* w64, const double* bc, double* partial,
-                                  int nblk, cudaStream_t st, const DcTabs* dc = nullptr);
+                                  cudaStream_t st, const DcTabs* dc = nullptr);
 cudaError_t launch_scat_update(int precision, const void* I, int64_t N, int G, int nd, const double* w64, const double* vol,
                                const double* ks, const double* em, double* Jold, float2* cm32, double2* cm64,
                                unsigned long long* d_max, cudaStream_t st);

@@ -48,7 +48,7 @@ constexpr uint32_t quad_bytes() { return 32u * (4u * sizeof(real) + 8u); }
 
 // header of a round in C
 struct RoundHdr {
-    uint32_t ns, nfar, e_off, ring0;  // slices, far sources, E of the round / 256, ring slot of its first place
+    uint32_t ns, nfar, pad, ring0;  // slices, far sources, ring slot of its first place
 };
 // a task in C
 template <typename real>
@@ -432,7 +432,7 @@ __global__ void __launch_bounds__(128) k_dir_write(DirBuild a) {
     const uint32_t far0 = (uint32_t)a.R + (uint32_t)(r % (a.A + 1)) * (uint32_t)a.Fs;
     const uint32_t zero = (uint32_t)a.R + (uint32_t)(a.A + 1) * (uint32_t)a.Fs;
     if (threadIdx.x == 0)
-        *reinterpret_cast<RoundHdr*>(C) = RoundHdr{ns, nfar, eoff[0], ri.x * 32u % (uint32_t)a.R};
+        *reinterpret_cast<RoundHdr*>(C) = RoundHdr{ns, nfar, 0u, ri.x * 32u % (uint32_t)a.R};
     const float4 om = a.om32[d], oml = a.om32lo[d];
     for (uint32_t k = warp; k < ns; k += 4) {
         const int nq = (int)a.nq[(size_t)d * a.SC + ri.x + k];

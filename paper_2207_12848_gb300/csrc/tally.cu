@@ -576,8 +576,7 @@ cudaError_t launch_prep_adjoint_src(int64_t N, int G, const double* vol, const d
 
 cudaError_t launch_tally(int precision, const void* I, int64_t N, int G, int nd, int d0, const double* w64,
                          double wsum, const double* vol, const double* ka, const double* em, double* J, double* Gam,
-                         double* partial, int nblk_, cudaStream_t st) {
-    (void)nblk_;
+                         double* partial, cudaStream_t st) {
     unsigned b = nb(N * G);
     if (b == 0) b = 1;
     if (precision == 64)
@@ -588,9 +587,8 @@ cudaError_t launch_tally(int precision, const void* I, int64_t N, int G, int nd,
 }
 
 cudaError_t launch_boundary_tally(int precision, const DevMesh& m, const void* I, int G, int nd, int d0,
-                                  const double* om64, const double* w64, const double* bc, double* partial, int nblk_,
+                                  const double* om64, const double* w64, const double* bc, double* partial,
                                   cudaStream_t st, const DcTabs* dc) {
-    (void)nblk_;
     const DcTabs tabs = dc ? *dc : DcTabs();
     if (m.n_bcells <= 0) return cudaSuccess;
     const unsigned b = (unsigned)m.n_bcells;
