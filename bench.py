@@ -353,9 +353,9 @@ def run_ours(args, dist: Dist):
     alg_bytes = bpu * N * D * G
     peaks = measured_peaks()
     achieved = alg_bytes / avg_launch_s / 1e9
-    from paper_2207_12848_gb300._lib import KERNELS
+    from paper_2207_12848_gb300._lib import kernel_name
     roof = {"bound": "hbm", "kernel": "%s (%s schedule, %d lanes per task)" % (
-                KERNELS.get(last.get("kernel_used", 0), "?"), {1: "level", 2: "dataflow"}.get(last["schedule_used"], "?"),
+                kernel_name(last), {1: "level", 2: "dataflow"}.get(last["schedule_used"], "?"),
                 last["lanes_used"]),
             "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s", "frac": achieved / peaks["hbm_gbs"],
             "peak_source": peaks["source"],
@@ -396,7 +396,7 @@ def run_ours(args, dist: Dist):
             tx = time.perf_counter() - t0
             swm = sx["t_sweep_ms"] / max(1, sx["sweep_launches"])
             extra[key] = {"value": sx["updates"] / tx, "unit": "updates/s", "ms_per_step": 1e3 * tx,
-                          "roofline": _roof(p, swm, peaks, KERNELS.get(sx["kernel_used"], "?"), law),
+                          "roofline": _roof(p, swm, peaks, kernel_name(sx), law),
                           "solve": {"it_pbc": sx["it_pbc"], "n_sweeps": sx["n_sweeps"], "defect": sx["defect"],
                                     "depth_max": sx["depth_max"], "depth_mean": sx["depth_mean"],
                                     "depth_max_scheme_a": last["depth_max"], "classify_ms": sx["t_classify_ms"],
@@ -547,7 +547,7 @@ def _roof_sweeps(p, sweep_ms_total: float, n_sweeps: int, updates: float, peaks:
 
 def _solve_entry(name: str, workload: str, p, ctx, stream, opts, steps: int, warmup: int, peaks: dict) -> dict:
     import torch
-    from paper_2207_12848_gb300._lib import KERNELS
+    from paper_2207_12848_gb300._lib import kernel_name
     N, D, G = p.mesh.n_cells, p.n_dir, p.n_groups
     J = torch.empty((N, G), dtype=torch.float64, device="cuda")
     Gm = torch.empty_like(J)
@@ -558,7 +558,7 @@ def _solve_entry(name: str, workload: str, p, ctx, stream, opts, steps: int, war
     return {"config": name, "workload": workload, "n_cells": N, "n_dir": D, "n_groups": G, "steps": steps,
             "value": upd / dt, "unit": "updates/s", "ms_per_step": 1e3 * dt / steps,
             "dtype": "f64" if opts.precision == 64 else "f32",
-            "roofline": _roof(p, sweep_ms, peaks, KERNELS.get(st["kernel_used"], "?")) if st["sweep_launches"] else None,
+            "roofline": _roof(p, sweep_ms, peaks, kernel_name(st)) if st["sweep_launches"] else None,
             "solve": {"depth_max": st["depth_max"], "depth_mean": st["depth_mean"], "it_scat": st["it_scat"],
                       "it_pbc": st["it_pbc"], "n_sweeps": st["n_sweeps"], "defect": st["defect"],
                       "classify_ms": st["t_classify_ms"], "levelise_ms": st["t_levelise_ms"],
@@ -627,7 +627,7 @@ def adjoint_entry(args, stream, peaks: dict, steps: int, warmup: int, cpu: bool 
 
     import oracle
     from paper_2207_12848_gb300 import Context, default_opts
-    from paper_2207_12848_gb300._lib import KERNELS
+    from paper_2207_12848_gb300._lib import kernel_name
     p = make_problem("adjoint", rank, args.threads, args.cells)
     N, D, G = p.mesh.n_cells, p.n_dir, p.n_groups
     rng = np.random.default_rng(5)
@@ -652,16 +652,16 @@ def adjoint_entry(args, stream, peaks: dict, steps: int, warmup: int, cpu: bool 
         st = outs[-1]
         e = {"config": "5 (differentiation)", "workload": WORKLOADS["adjoint"], "n_cells": N, "n_dir": D,
              "n_groups": G, "steps": steps, "value": upd / dt, "unit": "updates/s", "ms_per_step": 1e3 * dt / steps,
-             "dtype": "f32", "roofline": _roof_sweeps(p, t_sw, sweeps, upd, peaks, KERNELS.get(st["kernel_used"], "?")),
+             "dtype": "f32", "roofline": _roof_sweeps(p, t_sw, sweeps, upd, peaks, kernel_name(st)),
              "gpu_launches": sum(o["kernel_launches"] for o in outs),
              "solve": {"depth_max": st["depth_max"], "forward_sweeps": st["it_scat"], "transposed_passes": st["it_pbc"],
                        "sweeps": st["n_sweeps"], "sweep_ms_per_launch": t_sw / max(1, sweeps),
                        "assemble_ms": st["t_assemble_ms"]}}
         e["forward_roofline"] = _roof(p, sf["t_sweep_ms"] / max(1, sf["sweep_launches"]), peaks,
-                                      KERNELS.get(sf["kernel_used"], "?"))
+                                      kernel_name(sf))
         n_tr = sum(o["it_pbc"] for o in outs)  # transposed passes
         e["transposed_roofline"] = _roof_sweeps(p, sum(o["t_transposed_ms"] for o in outs), n_tr,
-                                                float(N * D * 2 * G * n_tr), peaks, KERNELS.get(st["kernel_used"], "?"))
+                                                float(N * D * 2 * G * n_tr), peaks, kernel_name(st))
         # accuracy of the FP32 gradients against the FP64 adjoint of the same inputs
         gk64, ge64 = torch.empty_like(J), torch.empty_like(J)
         ctx.adjoint_dev(gk64, ge64, None, dg, default_opts(precision=64))
@@ -697,7 +697,7 @@ def adjoint_entry(args, stream, peaks: dict, steps: int, warmup: int, cpu: bool 
         s2, _ = ctx.solve_dev(J2, G2m, default_opts(precision=32))
         p2 = dataclasses.replace(p, kappa_abs=ka2, emissivity=em2)
         e["forward_roofline_2G"] = _roof(p2, s2["t_sweep_ms"] / max(1, s2["sweep_launches"]), peaks,
-                                         KERNELS.get(s2["kernel_used"], "?"))
+                                         kernel_name(s2))
     if cpu:
         # the oracle's adjoint (forward solve + transposed sweep) on the host cores, on a sample of directions
         cores = os.cpu_count() or 1

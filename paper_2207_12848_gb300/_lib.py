@@ -27,6 +27,16 @@ LAWS = {"balance": 0, "exp": 1}
 # forms of the batched sweep kernel (sweep_stats.kernel_used)
 KERNELS = {0: "none", 1: "k_plain", 2: "k_sweep", 3: "k_sweep_rec", 4: "k_sweep_op", 5: "k_sweep_op1", 6: "k_sweep_op2",
            7: "k_sweep_pk"}
+
+
+def kernel_name(stats: dict) -> str:
+    """The batched sweep's kernel by a solve's or adjoint's statistics (one block per direction reports as a packed sweep of
+    one lane and one block per SM)."""
+    if stats.get("kernel_used") == 7 and stats.get("lanes_used") == 1 and stats.get("blocks_per_sm_used") == 1:
+        return "k_sweep_dir"
+    return KERNELS.get(stats.get("kernel_used", 0), "?")
+
+
 OP_FORMATS = {"auto": 0, "lines": 1, "packets": 2}
 
 # every entry point include/sweep.h declares

@@ -1833,6 +1833,10 @@ sweep_status adjoint_impl(sweep_ctx* c, const sweep_opts* opts_in, const double*
     }
     S.updates_per_s = ttot > 0 ? S.updates / (ttot * 1e-3) : 0.0;
     S.schedule_used = plain ? SWEEP_SCHED_PLAIN : (tr_dir ? (int)SWEEP_SCHED_LEVEL : sched);
+    if (tr_dir) {  // as in a solve: what tells one block per direction from the packets
+        S.lanes_used = S.blocks_per_sm_used = 1;
+        S.threads_used = 64 * c->lev.dopt->W + 64;
+    }
     S.kernel_used = c->last_kernel;
     S.kernel_launches = (int32_t)(c->launches - launches0);
     if (stats) *stats = S;
