@@ -65,11 +65,11 @@ enum {
 };
 
 /* AUTO, with lanes_per_task, packets_per_step, block_threads and blocks_per_sm left at 0, op_format not LINES and
- * geometry_only 0, sweeps narrow levels (up to 256 tasks per direction and level on average, in FP64 512, or 96
- * with values of 4) with one block per direction: barriers between the levels of that direction only, and the operator in a stream of its
- * own order. Values of 1, 2 or 4 groups (transposed: 2 or 4 split groups), rows of up to 64 face sides, in FP64 the
- * BALANCE law. sweep_stats then reports schedule_used LEVEL, kernel_used PACKED, lanes_used and
- * blocks_per_sm_used 1. */
+ * geometry_only 0, sweeps narrow levels with one block per direction (up to 256 tasks per direction and level on
+ * average; in FP64 up to 512, or 160 with values of 4, fewer with few directions, several groups and cells of many sides):
+ * barriers between the levels of that direction only, and the operator in a stream of its own order. Values of 1, 2 or
+ * 4 groups (transposed: 2 or 4 split groups), rows of up to 64 face sides, in FP64 the BALANCE law. sweep_stats then
+ * reports schedule_used LEVEL, kernel_used PACKED, lanes_used and blocks_per_sm_used 1. */
 
 /* Absorption laws of the cell update (transport scheme (a) of Sec. 2.6, outflow = non-absorbed inflow
  * plus source; F_in = the inflow flux, P = the projected outflow area, tau = kappa_t V / P):

@@ -969,11 +969,25 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     // round takes. FP32: 204 tasks per level (2^18 cells, 64 directions) 1.21 against 1.60 ms for the packets of
     // all directions, 196 (scheme (b), 60 directions) 0.08 against 0.11 ms; 584 (2^21 cells, 128 directions) 9.7
     // against 10.6 ms, which the longer build does not earn back; 957 (25 meshes, 2 groups) 7.1 against
-    // 5.6 ms. FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. Four FP64 values
-    // leave room for three workers and a short ring: 92 tasks per level 10.4 against 12.3 ms (67,581 cells, 32 directions),
-    // 160 already 25.1 against 19.5. With more than two directions per SM the directions that wait cost more than the
-    // levels gain.
-    const double line = real_bytes == 4 ? 256.0 : (GC == 4 ? 96.0 : 512.0);
+    // 5.6 ms. With more than two directions per SM the directions that wait cost more than the levels gain.
+    // FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. A level costs the FP64 pipe of
+    // one SM time in proportion to its values and their entries, however few directions there are, while the mesh
+    // rows' level gets cheaper with fewer. Solves, ms by direction / over the mesh rows (tasks per level, directions), of
+    // 8,000 to 250,000 cells of 15.4 sides unless stated:
+    //   1 value   4.1 / 4.3 (263, 1)    4.3 / 5.4 (270, 4)    scheme (b) 0.58 / 0.58 (300, 1)    0.59 / 0.64 (331, 4)
+    //   2 values  4.87 / 4.86 (163, 1)  10.0 / 6.4 (263, 1)   5.3 / 6.0 (169, 4)   10.4 / 8.4 (270, 4)
+    //             5.3 / 7.2 (156, 12)   11.5 / 10.0 (249, 12)   11.1 / 13.9 (247, 32)
+    //             lattice 0.35 / 0.48 (197, 1)   scheme (b), n = 3 0.97 / 0.81 (300, 1)   1.02 / 1.15 (315, 12)
+    //   4 values  6.16 / 6.21 (74, 7)   8.4 / 7.4 (96, 7)   11.1 / 11.5 (114, 32)   13.2 / 12.4 (128, 32)
+    //             19.4 / 27.5 (154, 96)   scheme (b), n = 1 0.41 / 0.39 (151, 7)   0.42 / 0.50 (159, 32)
+    // Four values leave room for three workers and a short ring. The mesh rows' transposed sweep takes twice as long:
+    // gradients of two groups 22.8 / 23.7 (148, 7). The caps are the widest levels measured.
+    double line = 256.0;
+    if (real_bytes == 8) {
+        const double sides = std::min((double)m.S / m.N, L.transport > 0 ? std::max(8.0, 2.0 * L.transport + 2.0) : 64.0);
+        const double weight = (GC == 4 ? 5.2 : (GC == 2 ? 2.0 : 1.1)) * (sides + 5.0), slow = transposed ? 2.0 : 1.0;
+        line = std::min(GC == 4 ? 160.0 : std::min(512.0, slow * (280.0 + 20.0 * nd)), slow * (6400.0 + 210.0 * nd) / weight);
+    }
     if (width > line || nd > 2 * sms) return cudaSuccess;
     // one round per level where the workers suffice (FP64 sums are bound by the FP64 pipe: four warps fill it)
     P.W = std::min(real_bytes == 8 ? Form<NARROW>::W : Form<MID>::W, std::max(1, (int)(1.2 * (width / 32.0 + 0.5) + 0.5)));

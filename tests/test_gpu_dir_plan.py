@@ -119,18 +119,21 @@ def test_kept_operators_make_room(gpu_lib):
             assert np.array_equal(c.solve(precision=q)[0], J)
 
 
-@pytest.mark.parametrize("n,kind,by_dir", [(12, "lattice", True), (16, "lattice", True), (60000, "voronoi", True),
-                                           (60000, "periodic", True), (24, "lattice", False)])
-def test_fp64_four_values(gpu_lib, n, kind, by_dir):
-    # four FP64 values a task leave room for fewer workers from 77 tasks a level on, and lose above 96; forward (four
-    # groups) and transposed (two), against the mesh-row kernel
+@pytest.mark.parametrize("n,kind,n_dir,fwd,tr", [
+    (12, "lattice", 6, True, True), (16, "lattice", 6, True, True), (60000, "voronoi", 6, False, True),
+    (60000, "voronoi", 40, True, True), (60000, "periodic", 40, True, True), (24, "lattice", 6, False, False),
+    (24, "lattice", 200, False, False)])
+def test_fp64_four_values(gpu_lib, n, kind, n_dir, fwd, tr):
+    # four FP64 values a task leave room for fewer workers from 77 tasks a level on, and the line for them lies lower the
+    # fewer directions there are; forward (four groups) and transposed (two), against the mesh-row kernel. Levels of 51, 89,
+    # 97 to 100 and 197 tasks
     if kind == "lattice":
         m = lattice_mesh(n)
-        om, w = fibonacci_directions(6, seed=1)
+        om, w = fibonacci_directions(n_dir, seed=1)
         rng = np.random.default_rng(2)
         ka, em = rng.uniform(0.1, 2.0, (m.n_cells, 4)), rng.uniform(0.0, 1.0, (m.n_cells, 4))
     else:
-        p = configs.voronoi_small(n, n_dir=6, n_groups=4, seed=54, n_src=8, periodic_box=kind == "periodic")
+        p = configs.voronoi_small(n, n_dir=n_dir, n_groups=4, seed=54, n_src=8, periodic_box=kind == "periodic")
         m, om, w, ka, em = p.mesh, p.omega, p.weight, p.kappa_abs, p.emissivity
     it = dict(precision=64, tol_pbc=0.0, max_it_pbc=2, tol_scat=0.0, max_it_scat=2)
     with Context(0) as c:
@@ -138,16 +141,32 @@ def test_fp64_four_values(gpu_lib, n, kind, by_dir):
         c.set_directions(om, w)
         c.set_material(ka, em)
         J, _, st, _ = c.solve(**it)
-        assert (st["lanes_used"] == 1 and st["blocks_per_sm_used"] == 1) == by_dir
+        assert (st["lanes_used"] == 1 and st["blocks_per_sm_used"] == 1) == fwd
         J0 = c.solve(schedule="dataflow", **it)[0]
         assert np.max(np.abs(J - J0)) <= 1e-12 * np.max(J0)
         c.set_material(ka[:, :2].copy(), em[:, :2].copy())
         g = np.random.default_rng(4).normal(size=(m.n_cells, 2))
         a = c.adjoint(dl_dJ=g, allow_not_converged=True, **it)
         b = c.adjoint(dl_dJ=g, allow_not_converged=True, schedule="dataflow", **it)
-        assert a[-1]["schedule_used"] == (1 if by_dir else 2) and b[-1]["schedule_used"] == 2
+        assert a[-1]["schedule_used"] == (1 if tr else 2) and b[-1]["schedule_used"] == 2
         for x, y in zip(a[:2], b[:2]):
             assert np.max(np.abs(x - y)) <= 1e-12 * np.max(np.abs(y))
+
+
+@pytest.mark.parametrize("n_dir,G,by_dir", [(1, 1, False), (16, 1, True), (1, 2, False), (40, 2, True)])
+def test_fp64_few_directions(gpu_lib, n_dir, G, by_dir):
+    # 348 tasks a level: one block per direction pays where the mesh rows have many directions to sweep
+    m = lattice_mesh(32)
+    om, w = fibonacci_directions(n_dir, seed=1)
+    rng = np.random.default_rng(3)
+    with Context(0) as c:
+        c.set_mesh(m)
+        c.set_directions(om, w)
+        c.set_material(rng.uniform(0.1, 2.0, (m.n_cells, G)), rng.uniform(0.0, 1.0, (m.n_cells, G)))
+        J, _, st, _ = c.solve(precision=64)
+        assert (st["lanes_used"] == 1 and st["blocks_per_sm_used"] == 1) == by_dir
+        J0 = c.solve(precision=64, schedule="dataflow")[0]
+        assert np.max(np.abs(J - J0)) <= 1e-12 * np.max(J0)
 
 
 def test_levels_hold_no_more_than_their_arrays(gpu_lib):
