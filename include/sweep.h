@@ -66,7 +66,8 @@ enum {
 
 /* AUTO, with lanes_per_task, packets_per_step, block_threads and blocks_per_sm left at 0, op_format not LINES and
  * geometry_only 0, sweeps narrow levels with one block per direction (up to 256 tasks per direction and level on
- * average; in FP64 up to 512, or 160 with values of 4, fewer with few directions, several groups and cells of many sides):
+ * average, with 4 groups and fewer than 38 directions 180 plus two for each; in FP64 up to 512, or 160 with values of 4, fewer with
+ * few directions, several groups and cells of many sides):
  * barriers between the levels of that direction only, and the operator in a stream of its own order. Values of 1, 2 or
  * 4 groups (transposed: 2 or 4 split groups), rows of up to 64 face sides, in FP64 the BALANCE law. sweep_stats then
  * reports schedule_used LEVEL, kernel_used PACKED, lanes_used and blocks_per_sm_used 1. */

@@ -969,7 +969,9 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     // round takes. FP32: 204 tasks per level (2^18 cells, 64 directions) 1.21 against 1.60 ms for the packets of
     // all directions, 196 (scheme (b), 60 directions) 0.08 against 0.11 ms; 584 (2^21 cells, 128 directions) 9.7
     // against 10.6 ms, which the longer build does not earn back; 957 (25 meshes, 2 groups) 7.1 against
-    // 5.6 ms. With more than two directions per SM the directions that wait cost more than the levels gain.
+    // 5.6 ms. Four values are bound by the sums of one SM sooner than the packets by few directions: 1.01 against 1.13 ms
+    // (156 tasks, 12 directions), 1.71 against 1.57 (249, 12), 1.82 against 1.85 (247, 32). With more than two
+    // directions per SM the directions that wait cost more than the levels gain.
     // FP64 has the mesh-row kernel to beat: 350 (the 32^3 lattice) 0.40 against 0.54 ms. A level costs the FP64 pipe of
     // one SM time in proportion to its values and their entries, however few directions there are, while the mesh
     // rows' level gets cheaper with fewer. Solves, ms by direction / over the mesh rows (tasks per level, directions), of
@@ -982,7 +984,7 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
     //             19.4 / 27.5 (154, 96)   scheme (b), n = 1 0.41 / 0.39 (151, 7)   0.42 / 0.50 (159, 32)
     // Four values leave room for three workers and a short ring. The mesh rows' transposed sweep takes twice as long:
     // gradients of two groups 22.8 / 23.7 (148, 7). The caps are the widest levels measured.
-    double line = 256.0;
+    double line = GC == 4 && !transposed ? std::min(256.0, 180.0 + 2.0 * nd) : 256.0;
     if (real_bytes == 8) {
         const double sides = std::min((double)m.S / m.N, L.transport > 0 ? std::max(8.0, 2.0 * L.transport + 2.0) : 64.0);
         const double weight = (GC == 4 ? 5.2 : (GC == 2 ? 2.0 : 1.1)) * (sides + 5.0), slow = transposed ? 2.0 : 1.0;

@@ -6,7 +6,7 @@ import pytest
 import oracle
 from synth import configs
 from synth.fields import fibonacci_directions
-from synth.mesh import star_mesh
+from synth.mesh import lattice_mesh, star_mesh
 
 pytestmark = pytest.mark.gpu
 PACKED = 7
@@ -52,6 +52,20 @@ def test_auto_sweeps_by_direction(ctx, n, n_dir, G, kw):
     load(ctx, p)
     assert by_direction(ctx.solve(**kw)[2])
     assert not by_direction(ctx.solve(schedule="level", **kw)[2])
+
+
+@pytest.mark.parametrize("G,n_dir,by_dir", [(4, 2, False), (4, 16, True), (2, 2, True)])
+def test_four_groups_few_directions(ctx, G, n_dir, by_dir):
+    # 197 tasks a level; FP32 intensities are the packets' bit for bit on either side of the line
+    m = lattice_mesh(24)
+    om, w = fibonacci_directions(n_dir, seed=1)
+    rng = np.random.default_rng(3)
+    ctx.set_mesh(m)
+    ctx.set_directions(om, w)
+    ctx.set_material(rng.uniform(0.1, 2.0, (m.n_cells, G)), rng.uniform(0.0, 1.0, (m.n_cells, G)))
+    J, _, st, _ = ctx.solve()
+    assert by_direction(st) == by_dir
+    assert np.array_equal(J, ctx.solve(schedule="dataflow", packets_per_step=2)[0])
 
 
 @pytest.mark.parametrize("kind", ["vacuum", "periodic", "inflow"])
