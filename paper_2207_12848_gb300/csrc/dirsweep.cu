@@ -93,7 +93,8 @@ struct DirBuild {
     uint2* rtab;               // [nd][RC + 1] {C offset / 16, E offset / 256} of each round
     int2* tot;                 // [nd] slices, rounds
     DirMeta* meta;             // [nd]
-    int32_t* stat;             // [0] does not apply, [1] most far sources of a slice, [2] bound on a round's E bytes
+    int32_t* stat;             // [0] does not apply, [1] most far sources of a slice, [2] bound on a round's E bytes, [3] a level
+                               // is too wide for the ring
     uint32_t e_slot, quad_b;   // E bytes of a round's slot, bytes of a quad
     unsigned char *E, *C;
     const uint32_t* rowptr;
@@ -129,14 +130,15 @@ __device__ uint64_t entry_mask(const DirBuild& a, uint32_t c, int d, float* P) {
     return m;
 }
 
-// The plan's slots turned out too small for the E of a round: the host plans again with the bound, and until then
-// nothing more is counted (a second count of 2^18 cells, 128 directions costs 2.1 ms of a 15 ms solve).
 // Raises *p to v, by an atomic only where it would change it: of the hundreds of thousands of blocks and slices few do, and
 // atomics on one address come one after the other.
 __device__ __forceinline__ void raise_stat(int32_t* p, int v) {
     if (v > *(volatile int32_t*)p) atomicMax(p, v);
 }
-__device__ __forceinline__ bool slot_too_small(const DirBuild& a) { return (uint32_t)a.stat[2] > a.e_slot; }
+// The plan is over: its slots are too small for the E of a round, and the host plans again with the bound (a second count of
+// 2^18 cells, 128 directions costs 2.1 ms of a 15 ms solve), or a level is too wide for the ring (found after the count
+// it cost 90 us of a 0.7 ms solve: 8,000 cells, scheme (b), FP64).
+__device__ __forceinline__ bool plan_over(const DirBuild& a) { return a.stat[3] || (uint32_t)a.stat[2] > a.e_slot; }
 
 __device__ __forceinline__ int level_slices(int n) { return (n + 31) >> 5; }
 // A level of n slices has ceil(n / W) rounds of equal size, so its last round is not a small remainder.
@@ -173,9 +175,15 @@ __device__ int level_scan(int nl, int reverse, F v, int32_t* out) {
     return s_carry;
 }
 
-// First slice of every level.
+// A source that is not in the ring at its level's end was summed A rounds before any round of the level or earlier: the
+// fetch of the round, A iterations ahead of its sums, finds it in memory.
+__device__ __forceinline__ bool ring_too_short(const DirBuild& a, int ns) { return (ns + a.A * a.W) * 32 > a.R; }
+
+// First slice of every level, and whether the ring is long enough for it.
 __global__ void __launch_bounds__(1024) k_dir_slices(DirBuild a) {
     const int d = blockIdx.x;
+    for (int L = threadIdx.x; L < a.depth[d]; L += 1024)
+        if (ring_too_short(a, level_slices(a.dcnt[(size_t)d * a.cap + L]))) atomicOr(&a.stat[3], 1);
     const int32_t* cnt = a.dcnt + (size_t)d * a.cap;
     const int n = level_scan(a.depth[d], a.transposed, [&](int L) { return level_slices(cnt[L]); }, a.sbase + (size_t)d * a.lcap);
     if (threadIdx.x == 0) {
@@ -186,7 +194,7 @@ __global__ void __launch_bounds__(1024) k_dir_slices(DirBuild a) {
 
 // First round of every level.
 __global__ void __launch_bounds__(1024) k_dir_rounds(DirBuild a) {
-    if (slot_too_small(a)) return;
+    if (plan_over(a)) return;
     const int d = blockIdx.x;
     const int32_t* nr = a.nround + (size_t)d * a.lcap;
     const int n = level_scan(a.depth[d], a.transposed, [&](int L) { return nr[L]; }, a.rbase + (size_t)d * a.lcap);
@@ -215,7 +223,7 @@ __device__ int cut_rounds(const uint32_t* sfar, int ns, int per, uint32_t Fs, F 
 template <bool WRITE>
 __global__ void __launch_bounds__(128) k_dir_cut(DirBuild a) {
     const int L = blockIdx.x * 128 + threadIdx.x, d = blockIdx.y;
-    if (L >= a.depth[d] || slot_too_small(a)) return;
+    if (L >= a.depth[d] || plan_over(a)) return;
     const int ns = level_slices(a.dcnt[(size_t)d * a.cap + L]), s0 = a.sbase[(size_t)d * a.lcap + L];
     if (s0 + ns > a.SC) return;
     const uint32_t* sf = a.sfar + (size_t)d * a.SC + s0;
@@ -238,7 +246,7 @@ constexpr int PLACE_THREADS = 128;
 __global__ void __launch_bounds__(PLACE_THREADS) k_dir_place(DirBuild a) {
     __shared__ int s_bin[MAX_Q + 1], s_end[MAX_Q + 1], s_first;
     const int L = blockIdx.x, d = blockIdx.y;
-    if (L >= a.depth[d]) return;
+    if (L >= a.depth[d] || a.stat[3]) return;
     const int n = a.dcnt[(size_t)d * a.cap + L];
     const uint32_t* src = a.list + (size_t)d * a.N + a.dbase[(size_t)d * a.cap + L];
     const int s0 = a.sbase[(size_t)d * a.lcap + L], ns = level_slices(n);
@@ -300,13 +308,11 @@ __device__ __forceinline__ uint32_t near_slot(const DirBuild& a, int d, int32_t 
 // Far entries of each slice (one block per level of a direction, a warp per slice).
 __global__ void __launch_bounds__(128) k_dir_count(DirBuild a) {
     const int L = blockIdx.x, d = blockIdx.y;
-    if (L >= a.depth[d] || slot_too_small(a)) return;
+    if (L >= a.depth[d] || plan_over(a)) return;
     const int ns = level_slices(a.dcnt[(size_t)d * a.cap + L]), s0 = a.sbase[(size_t)d * a.lcap + L];
     if (s0 + ns > a.SC) return;
     const uint32_t end = (uint32_t)(s0 + ns) * 32u;
-    // a source that is not in the ring at its level's end was summed A rounds before any round of the level or
-    // earlier: the fetch of the round, A iterations ahead of its sums, finds it in memory
-    if (threadIdx.x == 0 && (ns + a.A * a.W) * 32 > a.R) atomicOr(&a.stat[0], 1);
+    if (threadIdx.x == 0 && ring_too_short(a, ns)) atomicOr(&a.stat[0], 1);  // a plan made again may have a shorter ring
     const int lane = threadIdx.x & 31;
     for (int k = threadIdx.x >> 5; k < ns; k += 4) {
         const size_t t = ((size_t)d * a.SC + s0 + k) * 32 + lane;
@@ -360,7 +366,7 @@ template <typename real>
 __global__ void __launch_bounds__(1024) k_dir_offsets(DirBuild a) {
     const int d = blockIdx.x;
     const int2 t = a.tot[d];
-    if (t.x > a.SC || t.y > a.RC || slot_too_small(a)) return;
+    if (t.x > a.SC || t.y > a.RC || plan_over(a)) return;
     const uint32_t* nq = a.nq + (size_t)d * a.SC;
     uint32_t* eoff = a.eoff + (size_t)d * (a.SC + 1);
     uint32_t* coff = a.coff + (size_t)d * (a.RC + 1);
@@ -1091,14 +1097,14 @@ cudaError_t dir_plan(const DevMesh& m, Levels& L, DirOp& P, bool transposed, int
         else k_dir_offsets<float><<<nd, 1024, 0, st>>>(a);
         k_dir_bases<<<1, 1024, 0, st>>>(P.meta, nd, total, (uint32_t*)(ws + o_sc));
         P.launches += attempt == 0 ? 8 : 6;
-        int32_t stat[3] = {};
+        int32_t stat[4] = {};
         int64_t tt[2] = {};
         if ((e = cudaMemcpyAsync(stat, a.stat, sizeof stat, cudaMemcpyDeviceToHost, st))) return e;
         if ((e = cudaMemcpyAsync(tt, total, sizeof tt, cudaMemcpyDeviceToHost, st))) return e;
         if ((e = cudaStreamSynchronize(st))) return e;
         P.e_bytes = tt[0];
         P.c_bytes = tt[1];
-        if (stat[0]) return cudaSuccess;
+        if (stat[0] || stat[3]) return cudaSuccess;
         // a round's E, and a slice's far sources, must fit their slots
         bool fits = true;
         if (stat[1] > P.Fs) {
