@@ -862,8 +862,10 @@ __global__ void __launch_bounds__(DIR_BOUND)
                 }
             };
             auto need = [&](int lim) {  // rounds below lim have arrived
-                for (; ok && wt < min(lim, nr); ++wt) {
+                while (ok && wt < min(lim, nr)) {
                     ok = wt < iss && mbar_wait(&bar[ws], ph, a.spin_budget);
+                    if (!ok) break;  // the place stays at the round that has not arrived
+                    ++wt;
                     ws = ws + 1 == depth ? 0u : ws + 1;
                     ph ^= ws == 0 ? 1u : 0u;
                 }
@@ -887,11 +889,6 @@ __global__ void __launch_bounds__(DIR_BOUND)
             }
             if (on && *fail <= nr) {  // a bounded wait gave up: report, let the copies in flight land (the one waited for first)
                 atomicCAS(a.err, DEV_OK, DEV_TIMEOUT);
-                if (!ok) {  // back to the round whose wait gave up
-                    ph ^= ws == 0 ? 1u : 0u;
-                    ws = ws == 0 ? depth - 1 : ws - 1;
-                    --wt;
-                }
                 for (; wt < iss; ++wt) {
                     mbar_wait(&bar[ws], ph, a.spin_budget);
                     ws = ws + 1 == depth ? 0u : ws + 1;
