@@ -78,6 +78,7 @@ class sweep_stats(ctypes.Structure):
 
 
 _LIB = None
+_RAW_STREAM = None  # torch's handle of a device's current stream, looked up at the first call with tensors
 
 
 def load(path: str | None = None):
@@ -198,18 +199,22 @@ class Context:
             raise SweepError(st, self.lib.sweep_last_error(self.h).decode())
         return st
 
-    def _order(self, call):
-        """Runs a call that reads or writes CUDA tensors on the context's stream, ordered after what torch's current stream has
+    def _order(self, call, *args):
+        """A call that reads or writes CUDA tensors on the context's stream, ordered after what torch's current stream has
         still to do to them and before what it does next (the tensors' memory may be reused by it as soon as they are freed)."""
-        import torch
+        global _RAW_STREAM
+        if _RAW_STREAM is None:
+            import torch
+            _RAW_STREAM = torch._C._cuda_getCurrentRawStream
         # the raw handle first: a Stream object costs 2 us of a 240 us solve, twice a call
-        if torch._C._cuda_getCurrentRawStream(self.device) == self.stream:
-            return call()
+        if _RAW_STREAM(self.device) == self.stream:
+            return call(*args)
+        import torch
         cur = torch.cuda.current_stream(self.device)
         own = torch.cuda.ExternalStream(self.stream, self.device) if self.stream else torch.cuda.default_stream(self.device)
         own.wait_stream(cur)
         try:
-            return call()
+            return call(*args)
         finally:
             cur.wait_stream(own)
 
@@ -241,8 +246,8 @@ class Context:
         """Host arrays (numpy) or CUDA tensors (float64) of shape [n_cells, G], these of any stream that is current in torch."""
         if hasattr(kappa_abs, "is_cuda") and kappa_abs.is_cuda:
             G = kappa_abs.reshape(self.n_cells, -1).shape[1]
-            self._check(self._order(lambda: self.lib.sweep_set_material_dev(
-                self.h, G, _dp(kappa_abs), _dp(kappa_scat), _dp(emissivity), _dp(boundary_inflow))))
+            self._check(self._order(self.lib.sweep_set_material_dev, self.h, G, _dp(kappa_abs), _dp(kappa_scat),
+                                    _dp(emissivity), _dp(boundary_inflow)))
         else:
             ka = _host(kappa_abs, np.float64)
             ka = ka.reshape(ka.shape[0], -1) if ka.ndim > 1 else ka.reshape(-1, 1)
@@ -268,8 +273,8 @@ class Context:
         """Device outputs into CUDA float64 tensors [N,G]; returns (stats dict, status)."""
         o = opts or default_opts(**kw)
         st = sweep_stats()
-        s = self._check(self._order(lambda: self.lib.sweep_solve_dev(
-            self.h, ctypes.byref(o), _dp(J_out), _dp(Gamma_out), ctypes.byref(st))), (SWEEP_OK, SWEEP_NOT_CONVERGED))
+        s = self._check(self._order(self.lib.sweep_solve_dev, self.h, ctypes.byref(o), _dp(J_out), _dp(Gamma_out),
+                                    ctypes.byref(st)), (SWEEP_OK, SWEEP_NOT_CONVERGED))
         return st.as_dict(), s
 
     def rotate_directions(self, rotation, n_quad: int = 0):
@@ -308,7 +313,7 @@ class Context:
                     opts: sweep_opts | None = None, grad_kappa_scat_out=None, **kw):
         o = opts or default_opts(**kw)
         st = sweep_stats()
-        self._check(self._order(lambda: self.lib.sweep_adjoint_dev(
-            self.h, ctypes.byref(o), _dp(dl_dJ), _dp(dl_dGamma), _dp(grad_kappa_out), _dp(grad_emissivity_out),
-            _dp(grad_kappa_scat_out), ctypes.byref(st))))
+        self._check(self._order(self.lib.sweep_adjoint_dev, self.h, ctypes.byref(o), _dp(dl_dJ), _dp(dl_dGamma),
+                                _dp(grad_kappa_out), _dp(grad_emissivity_out), _dp(grad_kappa_scat_out),
+                                ctypes.byref(st)))
         return st.as_dict()
