@@ -862,10 +862,8 @@ __global__ void __launch_bounds__(DIR_BOUND)
                 }
             };
             auto need = [&](int lim) {  // rounds below lim have arrived
-                while (ok && wt < min(lim, nr)) {
+                for (; ok && wt < min(lim, nr); ++wt) {
                     ok = wt < iss && mbar_wait(&bar[ws], ph, a.spin_budget);
-                    if (!ok) break;  // the place stays at the round that has not arrived
-                    ++wt;
                     ws = ws + 1 == depth ? 0u : ws + 1;
                     ph ^= ws == 0 ? 1u : 0u;
                 }
@@ -889,10 +887,9 @@ __global__ void __launch_bounds__(DIR_BOUND)
             }
             if (on && *fail <= nr) {  // a bounded wait gave up: report, let the copies in flight land (the one waited for first)
                 atomicCAS(a.err, DEV_OK, DEV_TIMEOUT);
-                for (; wt < iss; ++wt) {
-                    mbar_wait(&bar[ws], ph, a.spin_budget);
-                    ws = ws + 1 == depth ? 0u : ws + 1;
-                    ph ^= ws == 0 ? 1u : 0u;
+                for (int w = ok ? wt : wt - 1; w < iss; ++w) {  // from the round whose wait gave up
+                    const uint32_t q = base + (uint32_t)w;
+                    mbar_wait(&bar[q % depth], q / depth & 1u, a.spin_budget);
                 }
             }
             __syncwarp();
